@@ -151,9 +151,8 @@ size_t glemur_workspace_bytes(int nx, int ny, int nz, int precision);
  * Kernel selection happens here, once per context; these environment
  * variables, read at this call, override it (all results stay within the
  * same tolerances):
- *   GLEMUR_TMA=0          mixed precision: register-staged tile loads even
- *                         where TMA tiles apply (nx a multiple of 4, nx >= 40,
- *                         ny >= 12)
+ *   GLEMUR_TMA=0          mixed precision: plain tile copies even where TMA
+ *                         tiles apply (nx a multiple of 4)
  *   GLEMUR_F64_FUSED=1    FP64: single-kernel mimetic stages (halo
  *                         recomputation) instead of the two-pass stages
  *   GLEMUR_KZ=k           z-planes per CTA of the stage kernels instead of

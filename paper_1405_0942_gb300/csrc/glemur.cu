@@ -19,7 +19,8 @@
 namespace glemur {
 cudaError_t launch_f64_mimetic(const StageArgs<double>& a, int stage, dim3 grid, cudaStream_t s);
 cudaError_t launch_f64_direct(const StageArgs<double>& a, int stage, dim3 grid, cudaStream_t s);
-cudaError_t launch_f32_mimetic(const StageArgs<float>& a, int stage, dim3 grid, cudaStream_t s);
+cudaError_t launch_f32_mimetic(const StageArgs<float>& a, const TmaMaps* maps, int stage,
+                               dim3 grid, cudaStream_t s);
 cudaError_t launch_f32_direct(const StageArgs<float>& a, int stage, dim3 grid, cudaStream_t s);
 cudaError_t prepare_f64_mimetic();
 cudaError_t prepare_f64_direct();
@@ -27,13 +28,10 @@ cudaError_t prepare_f32_mimetic();
 cudaError_t prepare_f32_direct();
 int ctas_per_sm_f64_mimetic();
 int ctas_per_sm_f64_direct();
-int ctas_per_sm_f32_mimetic();
+int ctas_per_sm_f32_mimetic(bool tma);
+int tile_rows_f32_mimetic();
+int tile_cols_f32_mimetic();
 int ctas_per_sm_f32_direct();
-cudaError_t launch_f32_mimetic_tma(const StageArgs<float>& a, const TmaMaps& maps, int stage,
-                                   dim3 grid, cudaStream_t s);
-cudaError_t prepare_f32_mimetic_tma();
-int ctas_per_sm_f32_mimetic_tma();
-int tile_rows_f32_mimetic_tma();
 
 cudaError_t launch_f64_split(const SplitArgs& a, int stage, cudaStream_t s, int curl);
 void split_ctas_per_sm(int b[6], int c[6], int curl);
@@ -201,6 +199,7 @@ struct glemur_ctx {
   double* dtlog;    // ring of GLEMUR_DT_LOG accepted step sizes
   int split;                             // FP64 mimetic stages in two passes
   int tma;                               // mixed mimetic stages with TMA tiles
+  int early;                             // stage grids that leave room for the next
   int tma_test;                          // test hook: unsatisfiable tile wait
   TmaMaps maps;                          // their tensor maps
   void* ys[2];                           // mimetic stages: stage inputs y_1..y_5
@@ -390,11 +389,12 @@ int elementwise_blocks(long long n) {
   return (int)(b < 4096 ? (b < 1 ? 1 : b) : 4096);
 }
 
-// Planes per CTA along z.  Cost model: the time of the busiest SM, in units
-// of one B plane (a CTA of kz planes computes kz + 2 B planes).  FP64 stages
-// are bound by the SM's FP64 pipe, which co-resident CTAs share, so an SM's
-// time is its CTA count x (kz + 2); the FP32 stages are latency-bound, so
-// up to `per_sm` co-resident CTAs overlap and the time is waves x (kz + 2).
+// Planes per CTA along z of the fused FP64 and the direct stage kernels.
+// Cost model: the time of the busiest SM, in units of one B plane (a CTA of
+// kz planes computes kz + 2 B planes).  FP64 stages are bound by the SM's
+// FP64 pipe, which co-resident CTAs share, so an SM's time is its CTA count x
+// (kz + 2); the FP32 stages are latency-bound, so up to `per_sm` co-resident
+// CTAs overlap and the time is waves x (kz + 2).
 int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe) {
   const char* env = getenv("GLEMUR_KZ");
   if (env && atoi(env) > 0) return atoi(env) < nz ? atoi(env) : nz;
@@ -407,6 +407,36 @@ int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe) {
     const long long slots = shared_pipe ? nsm : (long long)nsm * per_sm;
     const double waves = (double)((ctas + slots - 1) / slots);
     const double cost = waves * (kz + 2);
+    if (cost < best_cost - 1e-9) {
+      best_cost = cost;
+      best = kz;
+    }
+  }
+  return best;
+}
+
+// Planes per CTA along z of the mixed mimetic stage.  A CTA of kz planes runs
+// kz + 2 iterations and its prologue takes about half of one.  While all
+// CTAs are resident the time is that of the SM with the most: an iteration
+// takes 0.73 as long alone on an SM as beside a second CTA (128^3: kz = 15,
+// two CTAs per SM, 255 us an attempt; kz = 32, one, 386 us before the barrier
+// was split, 277 us beside it).  Beyond one wave CTAs start as others end and
+// the last ones leave about half a wave idle (128^3: kz = 8, 13 with 1.7,
+// 1.05 waves 291, 325 us).  Long marches lose to short ones on grids of many
+// waves (384^3: kz = 28, 36, 48 take 4.89, 4.85, 4.91 ms, 192 takes 9 % more
+// than 32), hence the limit of 40.
+int choose_kz_march(int nz, int gxy, int nsm, int per_sm) {
+  const char* env = getenv("GLEMUR_KZ");
+  if (env && atoi(env) > 0) return atoi(env) < nz ? atoi(env) : nz;
+  if (nsm < 1) nsm = 1;
+  if (per_sm < 1) per_sm = 1;
+  int best = nz;
+  double best_cost = 1e300;
+  for (int kz = 1; kz <= nz && kz <= 40; ++kz) {
+    const long long ctas = (long long)gxy * ((nz + kz - 1) / kz);
+    const double waves = (double)ctas / ((double)nsm * per_sm);
+    const double load = ctas <= nsm ? 0.73 : (waves <= 1.0 ? 1.0 : waves + 0.5);
+    const double cost = load * (kz + 2.5);
     if (cost < best_cost - 1e-9) {
       best_cost = cost;
       best = kz;
@@ -439,6 +469,7 @@ StageArgs<T> make_args(const glemur_ctx* c, int stage, int diag, int force) {
   a.st = c->st;
   a.part = c->part;
   a.nblocks = c->nblocks;
+  a.early = c->early;
   a.tma_test = c->tma_test;
   return a;
 }
@@ -491,8 +522,7 @@ cudaError_t launch_stage(const glemur_ctx* c, int curl, int stage, int diag, int
       a.nblocks = c->nblocks_direct;
       return launch_f32_direct(a, stage, g, c->s);
     }
-    if (c->tma) return launch_f32_mimetic_tma(a, c->maps, stage, g, c->s);
-    return launch_f32_mimetic(a, stage, g, c->s);
+    return launch_f32_mimetic(a, c->tma ? &c->maps : nullptr, stage, g, c->s);
   }
   StageArgs<double> a = make_args<double>(c, stage, diag, force);
   a.k6 = (double*)k6;
@@ -678,13 +708,14 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 // 4-D map (x, y, z, component) of an FP32 SoA field with boxes of
-// YW x box_h x 1 x 3; out-of-range elements read as zero.
+// (tile width + 8) x box_h x 1 x 3; out-of-range elements read as zero.
 bool encode_field_map(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* m, void* base,
                       int nx, int ny, int nz, int box_h) {
   const cuuint64_t dims[4] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz, 3};
   const cuuint64_t strides[3] = {(cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4,
                                  (cuuint64_t)nx * ny * nz * 4};
-  const cuuint32_t box[4] = {(cuuint32_t)YW, (cuuint32_t)box_h, 1, 3};
+  const cuuint32_t box[4] = {(cuuint32_t)(tile_cols_f32_mimetic() + 8),
+                             (cuuint32_t)box_h, 1, 3};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -693,11 +724,11 @@ bool encode_field_map(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* m, voi
 }
 
 // TMA tiles for the mixed mimetic stages: rows 16-byte aligned (nx a
-// multiple of 4) and a grid at least one box wide and high (box heights:
-// tile height + 4 for the stage input, + 2 for B0).
+// multiple of 4; box heights: tile height + 4 for the stage input, + 2 for
+// B0).
 bool setup_tma(glemur_ctx* c) {
-  const int th = tile_rows_f32_mimetic_tma();
-  if (c->o.precision != GLEMUR_MIXED || c->nx % 4 || c->nx < YW || c->ny < th + 4) return false;
+  const int th = tile_rows_f32_mimetic();
+  if (c->o.precision != GLEMUR_MIXED || c->nx % 4) return false;
   const char* env = getenv("GLEMUR_TMA");
   if (env && atoi(env) == 0) return false;
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
@@ -913,26 +944,26 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   // status without any fault
   const char* tt = getenv("GLEMUR_TEST_TMA_TIMEOUT");
   c->tma_test = tt && (atoi(tt) == 1 || atoi(tt) == 2) ? atoi(tt) : 0;
-  if (e == cudaSuccess && setup_tma(c)) {
-    e = prepare_f32_mimetic_tma();
-    c->tma = 1;
-  }
+  if (e == cudaSuccess && setup_tma(c)) c->tma = 1;
   if (e == cudaSuccess) e = mixed ? prepare_f32_direct() : prepare_f64_direct();
   if (e != cudaSuccess) {
     delete c;
     return GLEMUR_ERR_CUDA;
   }
   const int gx = (nx + TX - 1) / TX, gy = (ny + TY - 1) / TY;
-  // the TMA mimetic tile's height depends on its geometry
-  const int thm = c->tma ? tile_rows_f32_mimetic_tma() : TY;
-  const int gym = (ny + thm - 1) / thm;
-  const int pm = mixed ? (c->tma ? ctas_per_sm_f32_mimetic_tma()
-                                 : ctas_per_sm_f32_mimetic())
-                       : ctas_per_sm_f64_mimetic();
+  const int twm = mixed ? tile_cols_f32_mimetic() : TX;
+  const int thm = mixed ? tile_rows_f32_mimetic() : TY;
+  const int gxm = (nx + twm - 1) / twm, gym = (ny + thm - 1) / thm;
+  const int pm = mixed ? ctas_per_sm_f32_mimetic(c->tma != 0) : ctas_per_sm_f64_mimetic();
   const int pd = mixed ? ctas_per_sm_f32_direct() : ctas_per_sm_f64_direct();
-  c->kz = choose_kz(nz, gx * gym, c->nsm, pm, !mixed);
-  c->grid = dim3(gx, gym, (nz + c->kz - 1) / c->kz);
-  c->nblocks = gx * gym * (int)c->grid.z;
+  c->kz = mixed ? choose_kz_march(nz, gxm * gym, c->nsm, pm)
+                : choose_kz(nz, gxm * gym, c->nsm, pm, true);
+  c->grid = dim3(gxm, gym, (nz + c->kz - 1) / c->kz);
+  c->nblocks = gxm * gym * (int)c->grid.z;
+  // a grid that leaves room beside it for the next stage's lets that one
+  // start its prologue meanwhile (48^3: 59.6 -> 58.7 us an attempt); a larger
+  // one's waiting CTAs would hold the slots its own still need
+  c->early = mixed && 2LL * c->nblocks <= (long long)pm * c->nsm;
   if (c->split) {
     // per pass one wave of CTAs of 256 threads, each over an equal range of
     // node warps; the partials' stride is the larger grid
