@@ -18,16 +18,15 @@
 
 namespace glemur {
 cudaError_t launch_f64_mimetic(const StageArgs<double>& a, int stage, dim3 grid, cudaStream_t s);
-cudaError_t launch_f64_direct(const StageArgs<double>& a, int stage, dim3 grid, cudaStream_t s);
+cudaError_t launch_f64_direct(const SplitArgs& a, int stage, cudaStream_t s);
+void direct64_ctas_per_sm(int c[6]);
 cudaError_t launch_f32_mimetic(const StageArgs<float>& a, const TmaMaps* maps, int stage,
                                dim3 grid, cudaStream_t s);
 cudaError_t launch_f32_direct(const StageArgs<float>& a, int stage, dim3 grid, cudaStream_t s);
 cudaError_t prepare_f64_mimetic();
-cudaError_t prepare_f64_direct();
 cudaError_t prepare_f32_mimetic();
 cudaError_t prepare_f32_direct();
 int ctas_per_sm_f64_mimetic();
-int ctas_per_sm_f64_direct();
 int ctas_per_sm_f32_mimetic(bool tma);
 int tile_rows_f32_mimetic();
 int tile_cols_f32_mimetic();
@@ -213,6 +212,7 @@ struct glemur_ctx {
   int* persist_base;                     // counters to zero before each launch
   size_t persist_zero_bytes;
   int nblocks_direct, kz_direct;         // direct-current launches
+  int direct_grid[6] = {};               // FP64 direct grids (CTAs)
   dim3 grid, grid_direct;
   int nsm;
   int target_unbounded;                  // the device's step target is LLONG_MAX
@@ -389,7 +389,7 @@ int elementwise_blocks(long long n) {
   return (int)(b < 4096 ? (b < 1 ? 1 : b) : 4096);
 }
 
-// Planes per CTA along z of the fused FP64 and the direct stage kernels.
+// Planes per CTA along z of the fused FP64 and the mixed direct stage kernels.
 // Cost model: the time of the busiest SM, in units of one B plane (a CTA of
 // kz planes computes kz + 2 B planes).  FP64 stages are bound by the SM's
 // FP64 pipe, which co-resident CTAs share, so an SM's time is its CTA count x
@@ -478,8 +478,7 @@ int nblocks_of(const glemur_ctx* c, int curl) {
   return curl == GLEMUR_CURL_DIRECT ? c->nblocks_direct : c->nblocks;
 }
 
-cudaError_t launch_split(const glemur_ctx* c, int stage, int diag, int force, void* k6,
-                         int curl) {
+SplitArgs split_args(const glemur_ctx* c, int diag, int force) {
   SplitArgs a;
   a.nx = c->nx;
   a.ny = c->ny;
@@ -489,7 +488,7 @@ cudaError_t launch_split(const glemur_ctx* c, int stage, int diag, int force, vo
   a.d[1] = (const double*)c->dbuf[1];
   a.B0s = (const double*)c->B0s;
   for (int j = 0; j < 5; ++j) a.k[j] = (double*)c->k[j];
-  a.k[5] = (double*)k6;
+  a.k[5] = nullptr;
   a.ys[0] = (double*)c->ys[0];
   a.ys[1] = (double*)c->ys[1];
   a.Bb = c->Bb;
@@ -505,6 +504,13 @@ cudaError_t launch_split(const glemur_ctx* c, int stage, int diag, int force, vo
     a.grid_b[j] = c->split_grid_b[j];
     a.grid_c[j] = c->split_grid_c[j];
   }
+  return a;
+}
+
+cudaError_t launch_split(const glemur_ctx* c, int stage, int diag, int force, void* k6,
+                         int curl) {
+  SplitArgs a = split_args(c, diag, force);
+  a.k[5] = (double*)k6;
   return launch_f64_split(a, stage, c->s, curl == GLEMUR_CURL_NNN ? 2 : 0);
 }
 
@@ -524,40 +530,22 @@ cudaError_t launch_stage(const glemur_ctx* c, int curl, int stage, int diag, int
     }
     return launch_f32_mimetic(a, c->tma ? &c->maps : nullptr, stage, g, c->s);
   }
+  if (curl == GLEMUR_CURL_DIRECT) {
+    SplitArgs a = split_args(c, diag, force);
+    a.k[5] = (double*)k6;
+    a.nblocks = c->nblocks_direct;
+    for (int j = 0; j < 6; ++j) a.grid_c[j] = c->direct_grid[j];
+    return launch_f64_direct(a, stage, c->s);
+  }
   StageArgs<double> a = make_args<double>(c, stage, diag, force);
   a.k6 = (double*)k6;
-  if (curl == GLEMUR_CURL_DIRECT) {
-    a.kz = c->kz_direct;
-    a.nblocks = c->nblocks_direct;
-    return launch_f64_direct(a, stage, g, c->s);
-  }
   return launch_f64_mimetic(a, stage, g, c->s);
 }
 
 // n attempts in one persistent launch: the plane counters and the barrier
 // start from zero (the per-plane touch counts after them are kept).
 cudaError_t launch_attempts_persist(const glemur_ctx* c, int n) {
-  SplitArgs a;
-  a.nx = c->nx;
-  a.ny = c->ny;
-  a.nz = c->nz;
-  for (int i = 0; i < 3; ++i) a.h2[i] = 2.0 * c->h[i];
-  a.d[0] = (const double*)c->dbuf[0];
-  a.d[1] = (const double*)c->dbuf[1];
-  a.B0s = (const double*)c->B0s;
-  for (int j = 0; j < 5; ++j) a.k[j] = (double*)c->k[j];
-  a.k[5] = nullptr;
-  a.ys[0] = (double*)c->ys[0];
-  a.ys[1] = (double*)c->ys[1];
-  a.Bb = c->Bb;
-  a.rb = nullptr;
-  a.Gb = c->Gb;
-  a.diag = c->o.diag_each_attempt ? 1 : 0;
-  a.force = 0;
-  a.periodic = 0;
-  a.st = c->st;
-  a.part = c->part;
-  a.nblocks = c->nblocks;
+  SplitArgs a = split_args(c, c->o.diag_each_attempt ? 1 : 0, 0);
   for (int j = 0; j < 6; ++j) a.grid_b[j] = a.grid_c[j] = c->persist_grid;
   PersistArgs pa = c->pa;
   pa.n_attempts = n;
@@ -770,32 +758,13 @@ int ctx_recompute_stages_saved(glemur_ctx* c, double dt, void* k6, double* const
   k_set_dt<<<1, 1, 0, c->s>>>(c->st, dt, 0);
   cudaError_t e = cudaGetLastError();
   for (int s = 0; s < 6 && e == cudaSuccess; ++s) {
-    SplitArgs a;
-    a.nx = c->nx;
-    a.ny = c->ny;
-    a.nz = c->nz;
-    for (int i = 0; i < 3; ++i) a.h2[i] = 2.0 * c->h[i];
-    a.d[0] = (const double*)c->dbuf[0];
-    a.d[1] = (const double*)c->dbuf[1];
-    a.B0s = (const double*)c->B0s;
-    for (int j = 0; j < 5; ++j) a.k[j] = (double*)c->k[j];
+    SplitArgs a = split_args(c, 0, 1);  // not periodic: the adjoint refuses those
     a.k[5] = s == 5 ? (double*)k6 : nullptr;
     a.ys[0] = a.ys[1] = nullptr;
     if (s >= 1) a.ys[s & 1] = yS[s];
     if (s < 5) a.ys[(s + 1) & 1] = yS[s + 1];
     a.Bb = BS[s];
     a.rb = RS[s];
-    a.Gb = c->Gb;
-    a.diag = 0;
-    a.force = 1;
-    a.periodic = 0;  // the adjoint refuses periodic contexts (ctx_info)
-    a.st = c->st;
-    a.part = c->part;
-    a.nblocks = c->nblocks;
-    for (int j = 0; j < 6; ++j) {
-      a.grid_b[j] = c->split_grid_b[j];
-      a.grid_c[j] = c->split_grid_c[j];
-    }
     e = launch_f64_split(a, s, c->s, 0);
   }
   return cuda_rc(e);
@@ -945,7 +914,7 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   const char* tt = getenv("GLEMUR_TEST_TMA_TIMEOUT");
   c->tma_test = tt && (atoi(tt) == 1 || atoi(tt) == 2) ? atoi(tt) : 0;
   if (e == cudaSuccess && setup_tma(c)) c->tma = 1;
-  if (e == cudaSuccess) e = mixed ? prepare_f32_direct() : prepare_f64_direct();
+  if (e == cudaSuccess && mixed) e = prepare_f32_direct();
   if (e != cudaSuccess) {
     delete c;
     return GLEMUR_ERR_CUDA;
@@ -955,7 +924,6 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   const int thm = mixed ? tile_rows_f32_mimetic() : TY;
   const int gxm = (nx + twm - 1) / twm, gym = (ny + thm - 1) / thm;
   const int pm = mixed ? ctas_per_sm_f32_mimetic(c->tma != 0) : ctas_per_sm_f64_mimetic();
-  const int pd = mixed ? ctas_per_sm_f32_direct() : ctas_per_sm_f64_direct();
   c->kz = mixed ? choose_kz_march(nz, gxm * gym, c->nsm, pm)
                 : choose_kz(nz, gxm * gym, c->nsm, pm, true);
   c->grid = dim3(gxm, gym, (nz + c->kz - 1) / c->kz);
@@ -996,9 +964,22 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
       }
     }
   }
-  c->kz_direct = choose_kz(nz, gx * gy, c->nsm, pd, !mixed);
-  c->grid_direct = dim3(gx, gy, (nz + c->kz_direct - 1) / c->kz_direct);
-  c->nblocks_direct = gx * gy * (int)c->grid_direct.z;
+  if (mixed) {
+    c->kz_direct = choose_kz(nz, gx * gy, c->nsm, ctas_per_sm_f32_direct(), false);
+    c->grid_direct = dim3(gx, gy, (nz + c->kz_direct - 1) / c->kz_direct);
+    c->nblocks_direct = gx * gy * (int)c->grid_direct.z;
+  } else {
+    // one wave of CTAs over equal ranges of node warps, as the two passes
+    int od[6];
+    direct64_ctas_per_sm(od);
+    const long long need = (c->N + 255) / 256;
+    c->nblocks_direct = 1;
+    for (int s = 0; s < 6; ++s) {
+      const long long cd = (long long)od[s] * c->nsm;
+      c->direct_grid[s] = (int)(need < cd ? need : cd);
+      if (c->direct_grid[s] > c->nblocks_direct) c->nblocks_direct = c->direct_grid[s];
+    }
+  }
 
   // zero displacement (x = X), B0 and stage fields; boundary entries of the
   // stage fields stay zero for ever (line-tied nodes do not move)

@@ -1,0 +1,141 @@
+// What the dense FP64 kernels share (the two-pass stages and the direct
+// stage): node ranges of a one-wave grid, the loads, the per-CTA partials and
+// the output of a stage at a node.
+#pragma once
+
+#include "control.cuh"
+#include "stage_kernels.cuh"
+
+namespace glemur {
+
+// How the passes load data that another CTA of the same launch may have
+// written: the per-pass kernels use the read-only path (__ldg) -- each pass
+// only reads what earlier launches wrote -- while the persistent attempt
+// kernel, whose CTAs read each other's results within one launch, uses
+// ordinary (weak) global loads: the read-only path may keep lines from an
+// earlier pass, whereas weak loads that follow, in causality order, an
+// acquire that observed the writer's release must return the released
+// values (the PTX memory model; the waits below are exactly that pattern).
+// The loads are volatile asm so that the compiler neither merges loads of
+// one address from different passes nor moves them across the waits.
+struct LdRO {
+  __device__ static __forceinline__ double ld(const double* p) { return __ldg(p); }
+  __device__ static __forceinline__ double2 ld2(const double2* p) { return __ldg(p); }
+  __device__ static __forceinline__ int ldi(const int* p) { return *p; }
+};
+struct LdL2 {
+  __device__ static __forceinline__ double ld(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+  }
+  __device__ static __forceinline__ double2 ld2(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+  }
+  __device__ static __forceinline__ int ldi(const int* p) {
+    int v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+  }
+};
+
+// This CTA's node range: warps [W b / G, W (b+1) / G) of the W = N/32 node
+// warps (rounded up), as node indices [begin, end).
+__device__ __forceinline__ void cta_range(int N, int& begin, int& end) {
+  const long long W = (N + 31) / 32;
+  const long long w0 = W * blockIdx.x / gridDim.x, w1 = W * (blockIdx.x + 1) / gridDim.x;
+  begin = (int)(w0 * 32);
+  end = (int)(w1 * 32 < N ? w1 * 32 : N);
+}
+
+// Interior nodes enumerated densely: t in [0, (nx-2)(ny-2)(nz-2)) -> node.
+// A warp then holds 32 interior nodes, so the interior code (central
+// differences only) runs with no boundary lanes in it.
+__device__ __forceinline__ int interior_node(const SplitArgs& a, int t, int& i, int& j, int& k) {
+  const int nxi = a.nx - 2, nyi = a.ny - 2;
+  i = 1 + t % nxi;
+  const int r = t / nxi;
+  j = 1 + r % nyi;
+  k = 1 + r / nyi;
+  return (k * a.ny + j) * a.nx + i;
+}
+
+// This CTA's partial of kind `kind`; the slots of the partial stride beyond
+// this launch's grid are zeroed (neutral for the sums and for the maxima of
+// non-negative values), so a pass with fewer CTAs than the stride leaves no
+// stale slot behind.
+__device__ __forceinline__ void put_partial(const SplitArgs& a, int kind, double v) {
+  double* p = a.part + kind * a.nblocks;
+  p[blockIdx.x] = v;
+  for (int b = gridDim.x + blockIdx.x; b < a.nblocks; b += gridDim.x) p[b] = 0.0;
+}
+
+// a.b - c.d as one multiply and five FMAs (one FP64 instruction fewer than
+// two dot products and a subtraction)
+__device__ __forceinline__ double dot3_sub(const double a[3], const double b[3],
+                                           const double c[3], const double d[3]) {
+  double t = a[0] * b[0];
+  t = fma(a[1], b[1], t);
+  t = fma(a[2], b[2], t);
+  t = fma(-c[0], d[0], t);
+  t = fma(-c[1], d[1], t);
+  return fma(-c[2], d[2], t);
+}
+
+// Stage S's output at interior node n of plane k from its velocity u: k_S and
+// the next stage input y_{S+1} = d + sum_{j<=S} dt a_{S+1,j} k_j, or (S = 5)
+// the fifth-order update, the embedded error and k6.
+template <int S, class LD>
+__device__ __forceinline__ void split_emit(const SplitArgs& a, const double* d, double* dout,
+                                           double* ynext, const double an[5], int N, int n,
+                                           int k, const double u[3], Acc<double>& acc) {
+  constexpr bool FINAL = S == 5;
+  const DevState* st = a.st;
+  const int sz = a.nx * a.ny;
+  if (!FINAL) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      a.k[S][c * N + n] = u[c];
+      // next stage input y_{S+1} = d + sum_{j<=S} dt a_{S+1,j} k_j
+      double v = LD::ld(&d[c * N + n]);
+#pragma unroll
+      for (int jj = 0; jj < S; ++jj) v = fma(an[jj], LD::ld(&a.k[jj][c * N + n]), v);
+      v = fma(an[S], u[c], v);
+      ynext[c * N + n] = v;
+      // periodic in z: the ghost of an end plane holds the same
+      // displacement (its position differs by the period)
+      if (a.periodic && (k == 1 || k == a.nz - 2))
+        ynext[c * N + n + (k == 1 ? 1 : -1) * (a.nz - 2) * sz] = v;
+    }
+  } else {
+    const double b0 = LD::ld(&st->dtb[0]), b2 = LD::ld(&st->dtb[2]),
+                 b3 = LD::ld(&st->dtb[3]), b5 = LD::ld(&st->dtb[5]);
+    const double e0 = LD::ld(&st->dte[0]), e2 = LD::ld(&st->dte[2]),
+                 e3 = LD::ld(&st->dte[3]), e4 = LD::ld(&st->dte[4]),
+                 e5 = LD::ld(&st->dte[5]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double k1 = LD::ld(&a.k[0][c * N + n]), k3 = LD::ld(&a.k[2][c * N + n]),
+                   k4 = LD::ld(&a.k[3][c * N + n]), k5 = LD::ld(&a.k[4][c * N + n]);
+      double up = b0 * k1;
+      up = fma(b2, k3, up);
+      up = fma(b3, k4, up);
+      up = fma(b5, u[c], up);
+      double er = e0 * k1;
+      er = fma(e2, k3, er);
+      er = fma(e3, k4, er);
+      er = fma(e4, k5, er);
+      er = fma(e5, u[c], er);
+      const double dn = LD::ld(&d[c * N + n]) + up;
+      dout[c * N + n] = dn;
+      if (a.periodic && (k == 1 || k == a.nz - 2))
+        dout[c * N + n + (k == 1 ? 1 : -1) * (a.nz - 2) * sz] = dn;
+      acc.max_lam(fabs(er));
+      if (a.k[5]) a.k[5][c * N + n] = u[c];
+    }
+  }
+}
+
+}  // namespace glemur
