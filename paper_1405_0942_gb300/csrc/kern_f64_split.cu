@@ -259,76 +259,83 @@ __global__ void __launch_bounds__(256) k_split_B(const SplitArgs a) {
 // One octilateral loop of the next-nearest-neighbour current (section
 // "Next Nearest Neighbor Mimetic Approach") in the index surface spanned by
 // P and Q: the eight in-plane neighbours V_1..V_8 at (along P, along Q) =
-// (1,-1), (1,0), (1,1), (0,1), (-1,1), (-1,0), (-1,-1), (0,-1), positions
-// r_m taken relative to the node (displacement differences plus the label
-// offsets).  Returns twice the circulation and twice the vector area (the
-// common factor 1/2 cancels in M J = c):
+// (1,-1), (1,0), (1,1), (0,1), (-1,1), (-1,0), (-1,-1), (0,-1) with
+// positions r_m.  Returns twice the circulation and twice the vector area
+// (the common factor 1/2 cancels in M J = c):
 //   circulation with edge-mean B (eq. "current discrete", eight edges):
-//     sum_m (B_m + B_m+1)/2 . (r_m+1 - r_m) = sum_m B_m . (r_m+1 - r_m-1) / 2
-//   vector area (eq. "sum of eight triangles": four corner triangles plus the
-//   inner quadrilateral through V_2, V_4, V_6, V_8): a surface spanning the
-//   loop, so its vector area is the loop's, sum_m r_m x r_m+1 / 2.
-// The vertices stream through registers (three positions and one B live).
+//     sum_m (B_m + B_m+1)/2 . (r_m+1 - r_m) = sum_m B_m . e_m / 2 with
+//     e_m = r_m+1 - r_m-1;
+//   vector area (eq. "sum of eight triangles": four corner triangles plus
+//   the inner quadrilateral): a surface spanning the loop, so its vector area
+//   is the loop's, which the three quadrilaterals V_1 V_2 V_3 V_4, V_1 V_4
+//   V_5 V_8 and V_5 V_6 V_7 V_8 give as half the cross products of their
+//   diagonals: e_2 x e_3 + (r_5 - r_1) x (r_8 - r_4) + e_6 x e_7.
+// The pass is bound by the FP64 pipe, so everything is in the e_m: e_2..e_7
+// are differences of the displacement plus label offsets, r_5 - r_1 = e_2 +
+// e_4, r_8 - r_4 = e_5 + e_7, and the loop closes: e_8 = -(e_2 + e_4 + e_6),
+// e_1 = -(e_3 + e_5 + e_7).  81 FP64 instructions a loop, where positions
+// relative to the node and eight cross products took 128, and one reciprocal
+// for the solve's three divisions: 64^3, pass C of stage 3 217 -> 137 us; a
+// 65^3 attempt 1.55 -> 1.05 ms.
 template <int P, int Q, class LD>
 __device__ __forceinline__ void nnn_loop(const SplitArgs& a, const double* __restrict__ y,
-                                         int N, int n, const double yc[3], double& circ2,
-                                         double area2[3]) {
-  constexpr int OP[8] = {1, 1, 1, 0, -1, -1, -1, 0};
-  constexpr int OQ[8] = {-1, 0, 1, 1, 1, 0, -1, -1};
+                                         int N, int n, double& circ2, double area2[3]) {
   const int sp = P == 0 ? 1 : (P == 1 ? a.nx : a.nx * a.ny);
   const int sq = Q == 0 ? 1 : (Q == 1 ? a.nx : a.nx * a.ny);
   const double hp = 0.5 * a.h2[P], hq = 0.5 * a.h2[Q];
-  double r0[3], b0[3], r1[3], rp[3], rc[3], bc[3];
+  const int v[8] = {n + sp - sq, n + sp, n + sp + sq, n + sq,
+                    n - sp + sq, n - sp, n - sp - sq, n - sq};
+  double e2[3], e3[3], e4[3], e5[3], e6[3], e7[3];
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    const int nn = n + OP[m] * sp + OQ[m] * sq;
-    double rv[3], bv[3];
+  for (int c = 0; c < 3; ++c) {
+    double r[8];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      rv[c] = LD::ld(&y[c * N + nn]) - yc[c];
-      bv[c] = LD::ld(&a.Bb[c * N + nn]);
-    }
-    if (OP[m] != 0) rv[P] += OP[m] > 0 ? hp : -hp;
-    if (OQ[m] != 0) rv[Q] += OQ[m] > 0 ? hq : -hq;
-    if (m == 0) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) { r0[c] = rv[c]; b0[c] = bv[c]; }
-    } else {
-      // r_m-1 x r_m
-      const double* u = m == 1 ? r0 : rc;
-      if (m == 1) {
-        area2[0] = u[1] * rv[2] - u[2] * rv[1];
-        area2[1] = u[2] * rv[0] - u[0] * rv[2];
-        area2[2] = u[0] * rv[1] - u[1] * rv[0];
-      } else {
-        area2[0] = fma(u[1], rv[2], fma(-u[2], rv[1], area2[0]));
-        area2[1] = fma(u[2], rv[0], fma(-u[0], rv[2], area2[1]));
-        area2[2] = fma(u[0], rv[1], fma(-u[1], rv[0], area2[2]));
-      }
-      if (m >= 2) {  // the term of vertex m-1: B_m-1 . (r_m - r_m-2)
-        const double* w = m == 2 ? r0 : rp;
-        double t = bc[0] * (rv[0] - w[0]);
-        t = fma(bc[1], rv[1] - w[1], t);
-        t = fma(bc[2], rv[2] - w[2], t);
-        circ2 = m == 2 ? t : circ2 + t;
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if (m == 1) r1[c] = rv[c];
-        rp[c] = m == 1 ? r0[c] : rc[c];
-        rc[c] = rv[c];
-        bc[c] = bv[c];
-      }
-    }
+    for (int m = 0; m < 8; ++m) r[m] = LD::ld(&y[c * N + v[m]]);
+    e2[c] = r[2] - r[0];
+    e3[c] = r[3] - r[1];
+    e4[c] = r[4] - r[2];
+    e5[c] = r[5] - r[3];
+    e6[c] = r[6] - r[4];
+    e7[c] = r[7] - r[5];
   }
-  // close the loop: r_8 x r_1, and the terms of V_8 and V_1
-  area2[0] = fma(rc[1], r0[2], fma(-rc[2], r0[1], area2[0]));
-  area2[1] = fma(rc[2], r0[0], fma(-rc[0], r0[2], area2[1]));
-  area2[2] = fma(rc[0], r0[1], fma(-rc[1], r0[0], area2[2]));
+  e2[Q] += a.h2[Q];
+  e3[P] -= hp;
+  e3[Q] += hq;
+  e4[P] -= a.h2[P];
+  e5[P] -= hp;
+  e5[Q] -= hq;
+  e6[Q] -= a.h2[Q];
+  e7[P] += hp;
+  e7[Q] -= hq;
+  double f[3], g[3];  // r_5 - r_1, r_8 - r_4
 #pragma unroll
-  for (int c = 0; c < 3; ++c) circ2 = fma(bc[c], r0[c] - rp[c], circ2);
+  for (int c = 0; c < 3; ++c) {
+    f[c] = e2[c] + e4[c];
+    g[c] = e5[c] + e7[c];
+  }
 #pragma unroll
-  for (int c = 0; c < 3; ++c) circ2 = fma(b0[c], r1[c] - rc[c], circ2);
+  for (int c = 0; c < 3; ++c) {
+    const double* b = a.Bb + c * N;
+    const double m1 = g[c] + e3[c], m8 = f[c] + e6[c];  // -e_1, -e_8
+    circ2 = c == 0 ? LD::ld(&b[v[1]]) * e2[c] : fma(LD::ld(&b[v[1]]), e2[c], circ2);
+    circ2 = fma(LD::ld(&b[v[2]]), e3[c], circ2);
+    circ2 = fma(LD::ld(&b[v[3]]), e4[c], circ2);
+    circ2 = fma(LD::ld(&b[v[4]]), e5[c], circ2);
+    circ2 = fma(LD::ld(&b[v[5]]), e6[c], circ2);
+    circ2 = fma(LD::ld(&b[v[6]]), e7[c], circ2);
+    circ2 = fma(-LD::ld(&b[v[0]]), m1, circ2);
+    circ2 = fma(-LD::ld(&b[v[7]]), m8, circ2);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+    double t = e2[c1] * e3[c2];
+    t = fma(-e2[c2], e3[c1], t);
+    t = fma(e6[c1], e7[c2], t);
+    t = fma(-e6[c2], e7[c1], t);
+    t = fma(f[c1], g[c2], t);
+    area2[c] = fma(-f[c2], g[c1], t);
+  }
 }
 
 // The next-nearest-neighbour current at interior node n and B there: the
@@ -339,13 +346,10 @@ __device__ __forceinline__ void nnn_loop(const SplitArgs& a, const double* __res
 template <class LD>
 __device__ __forceinline__ void nnn_current(const SplitArgs& a, const double* __restrict__ y,
                                             int N, int n, double J[3], double B[3]) {
-  double yc[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) yc[c] = LD::ld(&y[c * N + n]);
   double M[3][3], cr[3];
-  nnn_loop<1, 2, LD>(a, y, N, n, yc, cr[0], M[0]);
-  nnn_loop<2, 0, LD>(a, y, N, n, yc, cr[1], M[1]);
-  nnn_loop<0, 1, LD>(a, y, N, n, yc, cr[2], M[2]);
+  nnn_loop<1, 2, LD>(a, y, N, n, cr[0], M[0]);
+  nnn_loop<2, 0, LD>(a, y, N, n, cr[1], M[1]);
+  nnn_loop<0, 1, LD>(a, y, N, n, cr[2], M[2]);
   double adj[3][3];  // adj[r] = a_{r+1} x a_{r+2}
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
@@ -355,10 +359,10 @@ __device__ __forceinline__ void nnn_current(const SplitArgs& a, const double* __
     adj[r][1] = u[2] * v[0] - u[0] * v[2];
     adj[r][2] = u[0] * v[1] - u[1] * v[0];
   }
-  const double detM = dot3(M[0], adj[0]);
+  const double rM = recip(dot3(M[0], adj[0]));
 #pragma unroll
   for (int c = 0; c < 3; ++c)
-    J[c] = (cr[0] * adj[0][c] + cr[1] * adj[1][c] + cr[2] * adj[2][c]) / detM;
+    J[c] = (cr[0] * adj[0][c] + cr[1] * adj[1][c] + cr[2] * adj[2][c]) * rM;
 #pragma unroll
   for (int c = 0; c < 3; ++c) B[c] = LD::ld(&a.Bb[c * N + n]);
 }
