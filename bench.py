@@ -56,14 +56,14 @@ MIN_TIMED_S = 1.0              # repeat the block of timed attempts until this
 # captured from (kernel_source_hash()); a workload without an entry, or one
 # whose kernels have changed since, reports null
 NCU_TRAFFIC = {
-    ("braid64", "fp64", "mimetic"): (58502016, "db5e1b8813f3"),
-    ("braid64", "fp64", "direct"): (31323178, "db5e1b8813f3"),
-    ("braid64", "fp64", "nnn"): (44149290, "db5e1b8813f3"),
-    ("periodic64", "fp64", "mimetic"): (58303573, "db5e1b8813f3"),
-    ("braid64", "mixed", "mimetic"): (15671893, "db5e1b8813f3"),
-    ("braid64", "mixed", "direct"): (15827712, "db5e1b8813f3"),
-    ("braid128", "mixed", "mimetic"): (152399061, "db5e1b8813f3"),
-    ("prod384", "mixed", "mimetic"): (4718079786, "db5e1b8813f3"),
+    ("braid64", "fp64", "mimetic"): (57730944, "633176018912"),
+    ("braid64", "fp64", "direct"): (31326890, "633176018912"),
+    ("braid64", "fp64", "nnn"): (44000170, "633176018912"),
+    ("periodic64", "fp64", "mimetic"): (57533269, "633176018912"),
+    ("braid64", "mixed", "mimetic"): (15672021, "633176018912"),
+    ("braid64", "mixed", "direct"): (15827456, "633176018912"),
+    ("braid128", "mixed", "mimetic"): (152441216, "633176018912"),
+    ("prod384", "mixed", "mimetic"): (4717954389, "633176018912"),
 }
 
 

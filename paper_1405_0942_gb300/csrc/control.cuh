@@ -87,25 +87,26 @@ __device__ __forceinline__ double fifth_root(double r) {
   if (!(r > 1e-30 && r < 1e30)) return pow(r, 0.2);
   const double y = (double)powf((float)r, 0.2f);
   const double y2 = y * y;
-  return 0.2 * (4.0 * y + r / (y2 * y2));
+  return 0.2 * fma(4.0, y, r * recip(y2 * y2));
 }
 
-// dt-scaled coefficients for step size dt, one entry per thread (the 36
-// a_sj and the 6 b_j, b_j - b*_j; threads >= 42 idle).
+// dt-scaled coefficients for step size dt: the 36 a_sj and the 6 b_j,
+// b_j - b*_j, shared out over the block's threads.
 __device__ __forceinline__ void set_coeffs_parallel(DevState* st, double dt) {
-  const int t = threadIdx.x;
-  if (t < 36) {
-    const int s = t / 6, j = t % 6;
-    const double v = dt * CK_A[s][j];
-    st->dta[s][j] = v;
-    st->dtaf[s][j] = (float)v;
-  } else if (t < 42) {
-    const int s = t - 36;
-    const double b = dt * CK_B5[s], e = dt * (CK_B5[s] - CK_B4[s]);
-    st->dtb[s] = b;
-    st->dte[s] = e;
-    st->dtbf[s] = (float)b;
-    st->dtef[s] = (float)e;
+  for (int t = threadIdx.x; t < 42; t += blockDim.x) {
+    if (t < 36) {
+      const int s = t / 6, j = t % 6;
+      const double v = dt * CK_A[s][j];
+      st->dta[s][j] = v;
+      st->dtaf[s][j] = (float)v;
+    } else {
+      const int s = t - 36;
+      const double b = dt * CK_B5[s], e = dt * (CK_B5[s] - CK_B4[s]);
+      st->dtb[s] = b;
+      st->dte[s] = e;
+      st->dtbf[s] = (float)b;
+      st->dtef[s] = (float)e;
+    }
   }
 }
 
@@ -114,38 +115,40 @@ __device__ __forceinline__ void set_coeffs_parallel(DevState* st, double dt) {
 // takes the decision from a snapshot of the control state (all loads
 // independent, then all stores); the block then writes the dt-scaled
 // coefficients of the next attempt in parallel.  `sh` holds 96 doubles.
-template <class LD>
+// `wait` returns once the attempt's last stage is complete: the snapshot and
+// the diagnostics (the first stage's partials) do not need it.
+template <class LD, class Wait>
 __device__ void control_block(DevState* st, const double* part, int nb, int diag,
-                              double* dtlog, double* sh) {
+                              double* dtlog, double* sh, Wait wait) {
   __shared__ double dt_next;
   __shared__ int go_on;
   if (LD::ldi(&st->status) != ST_OK ||
-      LD::ldll(&st->n_accept) >= LD::ldll(&st->target))
+      LD::ldll(&st->n_accept) >= LD::ldll(&st->target)) {
+    wait();
     return;
+  }
+  if (diag) finalize_diag<LD>(st, part, nb, sh);
+  const double dt = LD::ld(&st->dt), lambda0 = LD::ld(&st->lambda0),
+               safety = LD::ld(&st->safety);
+  const double shrink_min = LD::ld(&st->shrink_min), grow_max = LD::ld(&st->grow_max),
+               dt_min = LD::ld(&st->dt_min);
+  const double t = LD::ld(&st->t);
+  const int replay = LD::ldi(&st->replay), consec = LD::ldi(&st->consec),
+            max_rejects = LD::ldi(&st->max_rejects);
+  const int cur = LD::ldi(&st->cur);
+  const long long n_acc = LD::ldll(&st->n_accept), n_rej = LD::ldll(&st->n_reject);
+  wait();
+  const unsigned flags = LD::ldu(&st->flags);
   double m = 0.0;
   for (int b = threadIdx.x; b < nb; b += blockDim.x)
     m = nanmax(m, LD::ld(&part[PART_LAMBDA * nb + b]));
   for (int o = 16; o > 0; o >>= 1) m = nanmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  __syncthreads();
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = nanmax(m, sh[i]);
-    sh[95] = m;
-  }
-  __syncthreads();
-  if (diag) finalize_diag<LD>(st, part, nb, sh);
-  if (threadIdx.x == 0) {
-    const double lam = sh[95];
-    const double dt = LD::ld(&st->dt), lambda0 = LD::ld(&st->lambda0),
-                 safety = LD::ld(&st->safety);
-    const double shrink_min = LD::ld(&st->shrink_min), grow_max = LD::ld(&st->grow_max),
-                 dt_min = LD::ld(&st->dt_min);
-    const double t = LD::ld(&st->t);
-    const unsigned flags = LD::ldu(&st->flags);
-    const int replay = LD::ldi(&st->replay), consec = LD::ldi(&st->consec),
-              max_rejects = LD::ldi(&st->max_rejects);
-    const int cur = LD::ldi(&st->cur);
-    const long long n_acc = LD::ldll(&st->n_accept), n_rej = LD::ldll(&st->n_reject);
+    const double lam = m;
     int status = ST_OK;
     bool accept = false;
     double dtn = dt;
@@ -165,7 +168,7 @@ __device__ void control_block(DevState* st, const double* part, int nb, int diag
     } else if (replay) {
       accept = true;
     } else if (lam > lambda0) {
-      double fac = safety * fifth_root(lambda0 / lam);
+      double fac = safety * fifth_root(lambda0 * recip(lam));
       if (fac < shrink_min) fac = shrink_min;
       dtn = dt * fac;
       if (consec + 1 > max_rejects || dtn < dt_min) status = ST_DT_UNDERFLOW;
@@ -173,7 +176,7 @@ __device__ void control_block(DevState* st, const double* part, int nb, int diag
       accept = true;
       double fac = 1.0;
       if (lam < 0.5 * lambda0) {
-        fac = lam > 0.0 ? safety * fifth_root(lambda0 / lam) : grow_max;
+        fac = lam > 0.0 ? safety * fifth_root(lambda0 * recip(lam)) : grow_max;
         if (fac > grow_max) fac = grow_max;
       }
       dtn = dt * fac;

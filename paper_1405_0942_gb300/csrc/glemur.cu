@@ -19,7 +19,6 @@
 namespace glemur {
 cudaError_t launch_f64_mimetic(const StageArgs<double>& a, int stage, dim3 grid, cudaStream_t s);
 cudaError_t launch_f64_direct(const SplitArgs& a, int stage, cudaStream_t s);
-void direct64_ctas_per_sm(int c[6]);
 cudaError_t launch_f32_mimetic(const StageArgs<float>& a, const TmaMaps* maps, int stage,
                                dim3 grid, cudaStream_t s);
 cudaError_t launch_f32_direct(const StageArgs<float>& a, int stage, dim3 grid, cudaStream_t s);
@@ -33,8 +32,8 @@ int tile_cols_f32_mimetic();
 int ctas_per_sm_f32_direct();
 
 cudaError_t launch_f64_split(const SplitArgs& a, int stage, cudaStream_t s, int curl);
-void split_ctas_per_sm(int b[6], int c[6], int curl);
-int persist_ctas_per_sm(int curl);
+cudaError_t prepare_f64_split();
+cudaError_t prepare_f64_direct();
 cudaError_t launch_f64_persist(const SplitArgs& a, const PersistArgs& pa, int grid, int curl,
                                cudaStream_t s);
 
@@ -105,11 +104,12 @@ bool pdl_enabled() {
 
 // Eq. "time stepping" and the acceptance rule after each attempt (see
 // control.cuh), as a kernel of one CTA.
+// Its predecessor, the attempt's last stage, triggers it after its own wait,
+// so all earlier stages are complete when it starts.
 __global__ void k_control(DevState* st, const double* part, int nb, int diag, double* dtlog) {
   pdl_trigger();
-  pdl_wait();
   __shared__ double sh[96];
-  control_block<LdPlain>(st, part, nb, diag, dtlog, sh);
+  control_block<LdPlain>(st, part, nb, diag, dtlog, sh, [] { pdl_wait(); });
 }
 
 // ---- layout conversions at the boundary (float64 SoA fields) ----------
@@ -179,6 +179,11 @@ __global__ void k_to_f64(long long M, const T* __restrict__ src, double* __restr
 
 using namespace glemur;
 
+// Grid of a dense FP64 pass.
+struct DenseShape {
+  int grid, threads;
+};
+
 struct glemur_ctx {
   int nx, ny, nz;
   long long N;
@@ -203,16 +208,15 @@ struct glemur_ctx {
   TmaMaps maps;                          // their tensor maps
   void* ys[2];                           // mimetic stages: stage inputs y_1..y_5
   double* Bb;                            // split path: B
-  double* Gb;                            // split path: g_0, g_1, g_2
+  double* Gb;                            // split path: node records
   int max_blocks, nblocks, kz;          // mimetic-current launches
-  int split_grid_b[6] = {}, split_grid_c[6] = {};  // FP64 two-pass grids (CTAs)
+  DenseShape dense_b, dense_c, dense_direct;  // FP64 pass B, pass C, direct stage
   int persist;                           // whole attempts in one persistent launch
-  int persist_grid;                      // its CTAs (all resident)
+  int persist_grid, persist_threads;     // its CTAs (all resident)
   PersistArgs pa;                        // its plan and counters (workspace)
   int* persist_base;                     // counters to zero before each launch
   size_t persist_zero_bytes;
   int nblocks_direct, kz_direct;         // direct-current launches
-  int direct_grid[6] = {};               // FP64 direct grids (CTAs)
   dim3 grid, grid_direct;
   int nsm;
   int target_unbounded;                  // the device's step target is LLONG_MAX
@@ -223,6 +227,9 @@ namespace {
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 constexpr int PERSIST_MAX_CTAS = 16384;
+// The workspace holds the partials of at least this many CTAs (the dense
+// FP64 passes run up to one per SM).
+constexpr int DENSE_MIN_PARTIALS = 256;
 
 struct Layout {
   size_t field, stage, part, state, ptrs, dtlog, persist, split, total;
@@ -241,7 +248,7 @@ Layout layout(int nx, int ny, int nz, int precision) {
   L.field = align256((size_t)(3 * N) * es);
   L.stage = align256((size_t)(3 * N) * sizeof(double));
   const long long gx = (nx + TX - 1) / TX, gy = (ny + TY - 1) / TY;
-  L.max_blocks = (int)(gx * gy * nz);
+  L.max_blocks = (int)(gx * gy * nz > DENSE_MIN_PARTIALS ? gx * gy * nz : DENSE_MIN_PARTIALS);
   L.part = align256((size_t)NPART * L.max_blocks * sizeof(double));
   L.state = align256(sizeof(DevState));
   L.ptrs = 256;
@@ -255,7 +262,7 @@ Layout layout(int nx, int ny, int nz, int precision) {
   // two stage inputs (mimetic stages); FP64 also B and the node records
   // (differences and 1/det G) of the two-pass stages
   L.split = 2 * L.field + (precision == GLEMUR_FP64 ? align256((size_t)(3 * N) * 8) +
-                                                          align256((size_t)(10 * N) * 8)
+                                                          align256((size_t)(10 * (N + 31)) * 8)
                                                     : 0);
   L.total = 8 * L.field + L.stage + L.part + L.state + L.ptrs + L.dtlog + L.persist + L.split;
   return L;
@@ -263,34 +270,35 @@ Layout layout(int nx, int ny, int nz, int precision) {
 
 int cuda_rc(cudaError_t e) { return e == cudaSuccess ? GLEMUR_OK : GLEMUR_ERR_CUDA; }
 
-// Node range [begin, end) of CTA b of G over n items in whole warps, as the
-// two-pass kernels' cta_range computes it on the device.
+// Range [begin, end) of CTA b of G over n items in whole warps, as the
+// kernels' cta_range computes it on the device.
 void host_cta_range(long long n, int b, int G, long long& begin, long long& end) {
-  const long long W = (n + 31) / 32;
-  const long long w0 = W * b / G, w1 = W * (b + 1) / G;
-  begin = w0 * 32;
-  end = w1 * 32 < n ? w1 * 32 : n;
+  const WarpShare w = warp_share(n, G);
+  begin = 32LL * ((long long)b * w.each + (b < w.extra ? b : w.extra));
+  end = begin + 32LL * (w.each + (b < w.extra));
+  if (end > n) end = n;
+  if (begin > n) begin = n;
 }
 
-// Plane of boundary item t, in the order of the kernels' boundary_node:
-// the inner parts of the z, y and x faces, the edges along x, y and z, the
-// corners.
-int host_boundary_plane(int nx, int ny, int nz, long long t) {
-  const long long xi = nx - 2, yi = ny - 2, zi = nz - 2;
-  const long long fz = xi * yi, fy = xi * zi, fx = yi * zi;
-  if (t < 2 * fz) return t < fz ? 0 : nz - 1;
-  t -= 2 * fz;
-  if (t < 2 * fy) return 1 + (int)((t < fy ? t : t - fy) / xi);
-  t -= 2 * fy;
-  if (t < 2 * fx) return 1 + (int)((t < fx ? t : t - fx) / yi);
-  t -= 2 * fx;
-  if (t < 4 * xi) return ((t / xi) & 2) ? nz - 1 : 0;
-  t -= 4 * xi;
-  if (t < 4 * yi) return ((t / yi) & 2) ? nz - 1 : 0;
-  t -= 4 * yi;
-  if (t < 4 * zi) return 1 + (int)(t % zi);
-  t -= 4 * zi;
-  return (t & 4) ? nz - 1 : 0;
+// Plane of boundary item t, in the order of the kernels' boundary_node (the
+// inner parts of the z, y and x faces, the edges along x, y and z, the
+// corners, each group padded to whole warps); -1 for a group's idle lanes.
+int host_boundary_plane(int nx, int ny, int nz, int t) {
+  const int xi = nx - 2, yi = ny - 2, zi = nz - 2;
+  const int fz = xi * yi, fy = xi * zi, fx = yi * zi;
+  if (t < pad32(2 * fz)) return t >= 2 * fz ? -1 : (t < fz ? 0 : nz - 1);
+  t -= pad32(2 * fz);
+  if (t < pad32(2 * fy)) return t >= 2 * fy ? -1 : 1 + (t < fy ? t : t - fy) / xi;
+  t -= pad32(2 * fy);
+  if (t < pad32(2 * fx)) return t >= 2 * fx ? -1 : 1 + (t < fx ? t : t - fx) / yi;
+  t -= pad32(2 * fx);
+  if (t < pad32(4 * xi)) return t >= 4 * xi ? -1 : (((t / xi) & 2) ? nz - 1 : 0);
+  t -= pad32(4 * xi);
+  if (t < pad32(4 * yi)) return t >= 4 * yi ? -1 : (((t / yi) & 2) ? nz - 1 : 0);
+  t -= pad32(4 * yi);
+  if (t < pad32(4 * zi)) return t >= 4 * zi ? -1 : 1 + t % zi;
+  t -= pad32(4 * zi);
+  return t >= 8 ? -1 : ((t & 4) ? nz - 1 : 0);
 }
 
 // The persistent kernel's plan: per CTA the plane intervals of its pass-B
@@ -302,7 +310,7 @@ int host_boundary_plane(int nx, int ny, int nz, long long t) {
 bool persist_plan(glemur_ctx* c, int G) {
   const int nx = c->nx, ny = c->ny, nz = c->nz;
   if (G < 1 || G > PERSIST_MAX_CTAS) return false;
-  const long long N = c->N, NI = (long long)(nx - 2) * (ny - 2) * (nz - 2);
+  const long long NI = (long long)(nx - 2) * (ny - 2) * (nz - 2);
   const long long A = (long long)(nx - 2) * (ny - 2);
   int* h = new (std::nothrow) int[4 * (size_t)nz + 64 + (size_t)G * (2 * PERSIST_BI + 2)];
   if (!h) return false;
@@ -327,10 +335,11 @@ bool persist_plan(glemur_ctx* c, int G) {
       vc[0] = vb[0] = 1 + (int)(t0 / A);
       vc[1] = vb[1] = 1 + (int)((t1 - 1) / A);
     }
-    host_cta_range(N - NI, b, G, t0, t1);
+    host_cta_range(boundary_items(nx, ny, nz), G - 1 - b, G, t0, t1);  // in reverse
     int q = 1;
     for (long long t = t0; t < t1; ++t) {
-      const int pl = host_boundary_plane(nx, ny, nz, t);
+      const int pl = host_boundary_plane(nx, ny, nz, (int)t);
+      if (pl < 0) continue;
       if (q > 1) {
         int& lo = vb[2 * (q - 1)];
         int& hi = vb[2 * (q - 1) + 1];
@@ -445,6 +454,22 @@ int choose_kz_march(int nz, int gxy, int nsm, int per_sm) {
   return best;
 }
 
+// Grid of a dense FP64 pass over the interior nodes and, for pass B, the
+// boundary nodes (see split64.cuh): one CTA per SM of at most `most` threads
+// and no more groups of four warps than its share of node warps fills.
+DenseShape dense_shape(const glemur_ctx* c, bool boundary, int most) {
+  const long long ni = (long long)(c->nx - 2) * (c->ny - 2) * (c->nz - 2);
+  const long long warps =
+      (ni + 31) / 32 + (boundary ? boundary_items(c->nx, c->ny, c->nz) / 32 : 0);
+  const long long share = (warps + c->nsm - 1) / c->nsm;
+  DenseShape d;
+  const long long t = 128 * ((share + 3) / 4);
+  d.threads = (int)(t < most ? t : most);
+  const long long need = (warps + d.threads / 32 - 1) / (d.threads / 32);
+  d.grid = (int)(need < c->nsm ? need : c->nsm);
+  return d;
+}
+
 template <typename T>
 StageArgs<T> make_args(const glemur_ctx* c, int stage, int diag, int force) {
   StageArgs<T> a;
@@ -500,10 +525,17 @@ SplitArgs split_args(const glemur_ctx* c, int diag, int force) {
   a.st = c->st;
   a.part = c->part;
   a.nblocks = c->nblocks;
-  for (int j = 0; j < 6; ++j) {
-    a.grid_b[j] = c->split_grid_b[j];
-    a.grid_c[j] = c->split_grid_c[j];
-  }
+  a.grid_b = c->dense_b.grid;
+  a.threads_b = c->dense_b.threads;
+  a.grid_c = c->dense_c.grid;
+  a.threads_c = c->dense_c.threads;
+  const long long ni = (long long)(c->nx - 2) * (c->ny - 2) * (c->nz - 2);
+  a.inner_b = warp_share(ni, a.grid_b);
+  a.bound_b = warp_share(boundary_items(c->nx, c->ny, c->nz), a.grid_b);
+  a.inner_c = warp_share(ni, a.grid_c);
+  a.dx = fast_div(c->nx - 2);
+  a.dy = fast_div(c->ny - 2);
+  a.dz = fast_div(c->nz - 2);
   return a;
 }
 
@@ -534,7 +566,9 @@ cudaError_t launch_stage(const glemur_ctx* c, int curl, int stage, int diag, int
     SplitArgs a = split_args(c, diag, force);
     a.k[5] = (double*)k6;
     a.nblocks = c->nblocks_direct;
-    for (int j = 0; j < 6; ++j) a.grid_c[j] = c->direct_grid[j];
+    a.grid_c = c->dense_direct.grid;
+    a.threads_c = c->dense_direct.threads;
+    a.inner_c = warp_share(a.inner_c.n, a.grid_c);
     return launch_f64_direct(a, stage, c->s);
   }
   StageArgs<double> a = make_args<double>(c, stage, diag, force);
@@ -546,7 +580,10 @@ cudaError_t launch_stage(const glemur_ctx* c, int curl, int stage, int diag, int
 // start from zero (the per-plane touch counts after them are kept).
 cudaError_t launch_attempts_persist(const glemur_ctx* c, int n) {
   SplitArgs a = split_args(c, c->o.diag_each_attempt ? 1 : 0, 0);
-  for (int j = 0; j < 6; ++j) a.grid_b[j] = a.grid_c[j] = c->persist_grid;
+  a.grid_b = a.grid_c = c->persist_grid;
+  a.threads_b = c->persist_threads;
+  a.inner_b = a.inner_c = warp_share(a.inner_b.n, c->persist_grid);
+  a.bound_b = warp_share(a.bound_b.n, c->persist_grid);
   PersistArgs pa = c->pa;
   pa.n_attempts = n;
   // counters (2 nz ints) and the barrier (at 4 nz ints) start at zero
@@ -906,6 +943,8 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev);
   const bool mixed = o.precision == GLEMUR_MIXED;
   if (e == cudaSuccess) e = mixed ? prepare_f32_mimetic() : prepare_f64_mimetic();
+  if (e == cudaSuccess && !mixed) e = prepare_f64_split();
+  if (e == cudaSuccess && !mixed) e = prepare_f64_direct();
   c->tma = 0;
   // GLEMUR_TEST_TMA_TIMEOUT=1 (2) makes the TMA prologue wait (the first
   // wait inside the plane loop) also wait on a barrier that never completes,
@@ -919,6 +958,9 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
     delete c;
     return GLEMUR_ERR_CUDA;
   }
+  c->dense_b = dense_shape(c, true, DENSE_T);
+  c->dense_c = dense_shape(c, false, o.curl == GLEMUR_CURL_NNN ? DENSE_T2 : DENSE_T);
+  c->dense_direct = dense_shape(c, false, DENSE_T2);
   const int gx = (nx + TX - 1) / TX, gy = (ny + TY - 1) / TY;
   const int twm = mixed ? tile_cols_f32_mimetic() : TX;
   const int thm = mixed ? tile_rows_f32_mimetic() : TY;
@@ -933,19 +975,8 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   // one's waiting CTAs would hold the slots its own still need
   c->early = mixed && 2LL * c->nblocks <= (long long)pm * c->nsm;
   if (c->split) {
-    // per pass one wave of CTAs of 256 threads, each over an equal range of
-    // node warps; the partials' stride is the larger grid
-    int ob[6], oc[6];
-    split_ctas_per_sm(ob, oc, o.curl == GLEMUR_CURL_NNN ? 2 : 0);
-    const long long need = (c->N + 255) / 256;
-    c->nblocks = 1;
-    for (int s = 0; s < 6; ++s) {
-      const long long cb = (long long)ob[s] * c->nsm, cc = (long long)oc[s] * c->nsm;
-      c->split_grid_b[s] = (int)(need < cb ? need : cb);
-      c->split_grid_c[s] = (int)(need < cc ? need : cc);
-      c->nblocks = c->split_grid_b[s] > c->nblocks ? c->split_grid_b[s] : c->nblocks;
-      c->nblocks = c->split_grid_c[s] > c->nblocks ? c->split_grid_c[s] : c->nblocks;
-    }
+    // one CTA per SM; the partials' stride is the larger grid
+    c->nblocks = c->dense_b.grid > c->dense_c.grid ? c->dense_b.grid : c->dense_c.grid;
   }
   // whole attempts in one persistent launch (FP64 two-pass stages of the
   // loop currents, line-tied), on request: measured slower than the
@@ -954,14 +985,10 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   if (c->split && o.curl != GLEMUR_CURL_DIRECT && !o.periodic_z) {
     const char* pe = getenv("GLEMUR_PERSIST");
     if (pe && atoi(pe) == 1) {
-      const int per = persist_ctas_per_sm(o.curl == GLEMUR_CURL_NNN ? 2 : 0);
-      long long G = (long long)per * c->nsm;
-      const long long need = (c->N + 255) / 256;
-      if (G > need) G = need;
-      if (per >= 1 && persist_plan(c, (int)G)) {
-        c->persist = 1;
-        if (c->nblocks < (int)G) c->nblocks = (int)G;
-      }
+      const DenseShape& p = o.curl == GLEMUR_CURL_NNN ? dense_shape(c, true, DENSE_T2) : c->dense_b;
+      c->persist_threads = p.threads;
+      if (persist_plan(c, p.grid)) c->persist = 1;
+      if (c->nblocks < p.grid) c->nblocks = p.grid;
     }
   }
   if (mixed) {
@@ -969,16 +996,7 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
     c->grid_direct = dim3(gx, gy, (nz + c->kz_direct - 1) / c->kz_direct);
     c->nblocks_direct = gx * gy * (int)c->grid_direct.z;
   } else {
-    // one wave of CTAs over equal ranges of node warps, as the two passes
-    int od[6];
-    direct64_ctas_per_sm(od);
-    const long long need = (c->N + 255) / 256;
-    c->nblocks_direct = 1;
-    for (int s = 0; s < 6; ++s) {
-      const long long cd = (long long)od[s] * c->nsm;
-      c->direct_grid[s] = (int)(need < cd ? need : cd);
-      if (c->direct_grid[s] > c->nblocks_direct) c->nblocks_direct = c->direct_grid[s];
-    }
+    c->nblocks_direct = c->dense_direct.grid;
   }
 
   // zero displacement (x = X), B0 and stage fields; boundary entries of the

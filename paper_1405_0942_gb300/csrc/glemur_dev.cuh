@@ -102,11 +102,16 @@ struct StageArgs {
 // with launch_pdl: the next kernel of the stream may then be scheduled onto
 // SMs that the current one has left while its last CTAs still run.  Each
 // such kernel calls pdl_trigger() (its own successor may be scheduled once
-// all of its CTAs have started) and pdl_wait() before it reads or writes
-// anything an earlier kernel of the stream touches, DevState included:
-// griddepcontrol.wait returns once the preceding grids have completed and
-// their memory operations are visible.  Every path through such a kernel
-// passes pdl_wait(), so completion stays transitive along the stream.
+// all of its CTAs have started) and pdl_wait(): griddepcontrol.wait returns
+// once the preceding grids have completed and their memory operations are
+// visible.  Every path through such a kernel passes pdl_wait(), so
+// completion stays transitive along the stream.  Before it, a kernel reads
+// and writes nothing an earlier kernel of the stream touches, with one
+// exception: a stage after an attempt's first (its first pass counts as one)
+// and the step control trigger after their own pdl_wait(), so that when a
+// successor of theirs starts, everything before them is complete, and it may
+// read ahead of its wait what its immediate predecessor does not write (the
+// control state above all, which only the step control changes).
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -134,6 +139,35 @@ cudaError_t launch_pdl(void (*k)(Exp...), dim3 grid, dim3 block, size_t smem, cu
   return cudaLaunchKernelEx(&cfg, k, static_cast<Act&&>(args)...);
 }
 
+// Division of 0 <= n < 2^31 by a divisor fixed on the host, as a multiply and
+// a shift (Granlund & Montgomery, PLDI 1994): an integer division by a
+// variable takes some 25 instructions and 200 cycles of latency.
+struct FastDiv {
+  unsigned m;
+  int s, d;
+  __device__ __forceinline__ int div(int n) const {
+    return (int)((__umulhi((unsigned)n, m) + (unsigned)n) >> s);
+  }
+};
+inline FastDiv fast_div(int d) {
+  FastDiv f;
+  f.d = d;
+  f.s = 0;
+  while ((1ll << f.s) < d) ++f.s;
+  f.m = (unsigned)(((1ull << 32) * ((1ull << f.s) - (unsigned)d)) / (unsigned)d + 1);
+  return f;
+}
+
+// n items in whole warps over the CTAs of a grid: `each` warps a CTA, one
+// more for the first `extra` (host-side division, no 64-bit one per thread).
+struct WarpShare {
+  int n, each, extra;
+};
+inline WarpShare warp_share(long long n, int grid) {
+  const long long w = (n + 31) / 32;
+  return WarpShare{(int)n, (int)(w / grid), (int)(w % grid)};
+}
+
 // Arguments of the FP64 two-pass stages (pass B: B and 1/det G at every
 // node; pass C: current, k_s and the next stage input).
 struct SplitArgs {
@@ -146,18 +180,32 @@ struct SplitArgs {
                        // boundary entries hold the fixed boundary positions
   double* Bb;          // B, 3N
   double* rb;          // 1/det G, N, or null (then written to Gb only)
-  double* Gb;          // per interior node n, 10 doubles at Gb + 10 n
-                       // (16-byte aligned): g_0, g_1, g_2 (index-space
-                       // differences, 3 components each) and 1/det G --
-                       // written by pass B, read by pass C
+  double* Gb;          // per interior node 10 doubles: g_0, g_1, g_2
+                       // (index-space differences, 3 components each) and
+                       // 1/det G -- written by pass B, read by pass C
+                       // (node_record)
   int diag, force;
   int periodic;        // periodic in z: planes 0, nz-1 are ghosts of nz-2, 1
   DevState* st;
   double* part;        // [NPART][nblocks] per-CTA partials
   int nblocks;         // partial stride: the largest of the grids
-  int grid_b[6];       // CTAs of pass B of each stage
-  int grid_c[6];       // CTAs of pass C of each stage
+  int grid_b, threads_b;  // CTAs of pass B, threads of each
+  int grid_c, threads_c;  // of pass C (or the direct stage)
+  WarpShare inner_b, bound_b, inner_c;  // interior and boundary nodes of each
+  FastDiv dx, dy, dz;     // by nx - 2, ny - 2, nz - 2
 };
+// Most threads of a dense pass's CTA (one CTA per SM): 32 warps at 64
+// registers a thread, since the warps of a quarter come to the end of a node
+// together and wait for the next one's loads together, so fewer, fuller
+// rounds win (64^3, 12.25 node warps a quarter: 16, 24, 32 warps per SM take
+// 322, 320, 302 us an attempt; 129 x 97 x 75: 1034, 1019, 1020).  16 warps at
+// 128 for the next-nearest-neighbour pass C and the direct stage.
+constexpr int DENSE_T = 1024, DENSE_T2 = 512;
+// Dynamic shared memory none of them uses: more than half of an SM's, so
+// that two CTAs never share one (a programmatic launch fills an SM that fell
+// free with two where it can, and leaves another without: 33^3 99 against 90
+// us an attempt, 64^3 at 16 warps 486 against 338).
+constexpr int DENSE_SMEM = 118784;
 
 // The persistent FP64 attempt kernel's plan and synchronisation state
 // (workspace memory): per node plane, completion counters of pass B and
@@ -180,6 +228,15 @@ struct PersistArgs {
                         // stage 3, so waits on it give up (-1: off)
 };
 
+// Boundary nodes as pass B enumerates them (boundary_node): seven groups of
+// one stencil variant each, padded to whole warps.
+__host__ __device__ constexpr int pad32(int n) { return (n + 31) & ~31; }
+__host__ __device__ constexpr int boundary_items(int nx, int ny, int nz) {
+  return pad32(2 * (nx - 2) * (ny - 2)) + pad32(2 * (nx - 2) * (nz - 2)) +
+         pad32(2 * (ny - 2) * (nz - 2)) + pad32(4 * (nx - 2)) + pad32(4 * (ny - 2)) +
+         pad32(4 * (nz - 2)) + 32;
+}
+
 // What the on-demand diagnostics (diagnostics.cu) need of a context.
 struct DiagCtx {
   int nx, ny, nz;
@@ -196,6 +253,24 @@ struct DiagCtx {
 
 __device__ __forceinline__ long long nidx(int i, int j, int k, int nx, int ny) {
   return ((long long)k * ny + j) * nx + i;
+}
+
+// 1/v, FP64: Newton-Raphson refinement of the hardware approximation
+// rcp.approx.ftz.f64, y <- y + y (1 - v y): each step squares the relative
+// error (the classical iteration for reciprocals, e.g. Muller et al.,
+// Handbook of Floating-Point Arithmetic, ch. on Newton-Raphson division),
+// so two steps take the approximation to within an ulp or two of the
+// correctly rounded 1/v in 4 FMAs, where the IEEE division costs about 12
+// FP64-pipe instructions -- a quarter of the FP64 work of forming B.  NaN
+// propagates; 0 and subnormal v give NaN or inf, and every caller has
+// already flagged det <= 0 (or tested v > 0 and takes inf for a limit).
+__device__ __forceinline__ double recip(double v) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+  double e = fma(-v, y, 1.0);
+  y = fma(y, e, y);
+  e = fma(-v, y, 1.0);
+  return fma(y, e, y);
 }
 
 // max of two non-negative doubles that propagates NaN (of either sign),

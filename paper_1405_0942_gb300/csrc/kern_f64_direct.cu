@@ -2,16 +2,14 @@
 //
 // The classic current at a node needs first and second differences of x,
 // first differences of B0s and nothing another thread has formed, so a stage
-// is one dense pass over the interior nodes: a wave of exactly the CTAs the
-// SMs hold, each over an equal range of node warps, every value loaded from
-// the node's neighbours through L1 (19 points of the stage input, 7 of B0s).
-// It is bound by the FP64 pipe (two lanes per SM and cycle: a warp
-// instruction takes it 16 cycles), which such a grid keeps evenly busy on
-// every SM; on shared-memory tiles (32 x 8 columns, one CTA of 8 warps per SM
-// at 180-226 registers) 65^3 gave 135 CTAs to 152 SMs and a stage took
-// 244 us, the pipe's time for its instructions being 106.  65^3: an attempt
-// 1.51 -> 0.755 ms; 64^3: stage 3 152 -> 116 us.  128 registers, 2 CTAs per
-// SM.
+// is one dense pass over the interior nodes (split64.cuh), every value loaded
+// from the node's neighbours through L1 (19 points of the stage input, 7 of
+// B0s).  It is bound by the FP64 pipe, which the equal shares of node warps
+// keep evenly busy: 65^3, an attempt 1.51 ms on shared-memory tiles (32 x 8
+// columns, one CTA of 8 warps per SM at 180-226 registers: 135 CTAs for 152
+// SMs, a stage 244 us where the pipe's time for its instructions was 106),
+// 0.755 ms on two CTAs of 8 warps per SM, 0.697 ms on one of 16 (128
+// registers).
 #include "split64.cuh"
 
 namespace glemur {
@@ -101,13 +99,12 @@ __device__ __forceinline__ void direct_current(const SplitArgs& a, const double*
 }
 
 template <int S>
-__global__ void __launch_bounds__(256, 2) k_direct64(const SplitArgs a) {
-  pdl_wait();
+__global__ void __launch_bounds__(DENSE_T2, 1) k_direct64(const SplitArgs a) {
+  int cur;
+  if (!dense_start<S == 0>(a, cur)) return;
+  __shared__ double red[32];
   const DevState* st = a.st;
-  if (!a.force && (st->status != ST_OK || st->n_accept >= st->target)) return;
-  __shared__ double red[8];
   const int N = a.nx * a.ny * a.nz;
-  const int cur = st->cur;
   const double* d = a.d[cur];
   double* dout = const_cast<double*>(a.d[cur ^ 1]);
   const double* y = S == 0 ? d : a.ys[S & 1];
@@ -117,7 +114,7 @@ __global__ void __launch_bounds__(256, 2) k_direct64(const SplitArgs a) {
   for (int j = 0; j < 5; ++j) an[j] = S < 5 && j <= S ? st->dta[S < 5 ? S + 1 : 0][j] : 0.0;
   Acc<double> acc;
   int tb, te;
-  cta_range((a.nx - 2) * (a.ny - 2) * (a.nz - 2), tb, te);
+  cta_range(a.inner_c, tb, te);
   for (int t = tb + threadIdx.x; t < te; t += blockDim.x) {
     int i, j, k;
     const int n = interior_node(a, t, i, j, k);
@@ -152,27 +149,26 @@ __global__ void __launch_bounds__(256, 2) k_direct64(const SplitArgs a) {
 
 }  // namespace
 
-// CTAs of 256 threads per SM that each stage can hold.
-void direct64_ctas_per_sm(int c[6]) {
+// Let the stages ask for DENSE_SMEM.
+cudaError_t prepare_f64_direct() {
   void (*k[6])(const SplitArgs) = {k_direct64<0>, k_direct64<1>, k_direct64<2>,
                                    k_direct64<3>, k_direct64<4>, k_direct64<5>};
-  for (int s = 0; s < 6; ++s) {
-    c[s] = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c[s], k[s], 256, 0);
-    if (c[s] < 1) c[s] = 1;
-  }
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < 6 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(k[i], cudaFuncAttributeMaxDynamicSharedMemorySize, DENSE_SMEM);
+  return e;
 }
 
-// Launch stage `stage` on grid_c[stage] CTAs of 256 threads.
+// Launch stage `stage`.
 cudaError_t launch_f64_direct(const SplitArgs& a, int stage, cudaStream_t s) {
-  const dim3 g(stage >= 0 && stage < 6 ? a.grid_c[stage] : 1);
+  const dim3 g(a.grid_c), nt(a.threads_c);
   switch (stage) {
-    case 0: return launch_pdl(k_direct64<0>, g, dim3(256), 0, s, a);
-    case 1: return launch_pdl(k_direct64<1>, g, dim3(256), 0, s, a);
-    case 2: return launch_pdl(k_direct64<2>, g, dim3(256), 0, s, a);
-    case 3: return launch_pdl(k_direct64<3>, g, dim3(256), 0, s, a);
-    case 4: return launch_pdl(k_direct64<4>, g, dim3(256), 0, s, a);
-    case 5: return launch_pdl(k_direct64<5>, g, dim3(256), 0, s, a);
+    case 0: return launch_pdl(k_direct64<0>, g, nt, DENSE_SMEM, s, a);
+    case 1: return launch_pdl(k_direct64<1>, g, nt, DENSE_SMEM, s, a);
+    case 2: return launch_pdl(k_direct64<2>, g, nt, DENSE_SMEM, s, a);
+    case 3: return launch_pdl(k_direct64<3>, g, nt, DENSE_SMEM, s, a);
+    case 4: return launch_pdl(k_direct64<4>, g, nt, DENSE_SMEM, s, a);
+    case 5: return launch_pdl(k_direct64<5>, g, nt, DENSE_SMEM, s, a);
     default: return cudaErrorInvalidValue;
   }
 }

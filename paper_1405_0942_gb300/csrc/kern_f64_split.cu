@@ -17,72 +17,77 @@
 //            k_s and, pointwise, the next stage input
 //            y_{s+1} = d + sum_{j<=s} dt a_{s+1,j} k_j; the last stage
 //            writes the fifth-order update and the embedded error instead.
-// Pass C reads g_a (and 1/det G) as pass B stored them, interleaved per
-// node, rather than forming g_a again from the stage input's neighbours:
-// 12 fewer FP64 additions per interior node and stage for 80 bytes written
-// and read (five 16-byte accesses each way), which HBM (used at well under
-// a fifth of its bandwidth by these passes) absorbs.
-// Each pass runs one wave of CTAs (as many as fit on the SMs: each pass
-// sizes its own grid), each over a contiguous range of whole warps of
-// nodes: the FP64 pipe is per SM, so every SM gets the same number of
-// node-warps (to within one per CTA) and no SM idles while another finishes
-// a second round.  Each pass is launched as a programmatic dependent of the
-// one before it (launch_pdl), so its CTAs take the SMs the previous pass
-// leaves and start as soon as it ends; a grid of exactly the CTAs the SMs
-// hold cannot crowd one SM when it is placed that way.  The per-CTA
-// partials (Lambda, E_M, xi) keep the fused kernel's layout.
+// Pass C reads g_a (and 1/det G) as pass B stored them, side by side for a
+// warp's nodes, rather than forming g_a again from the stage input's
+// neighbours: 12 fewer FP64 additions per interior node and stage for 80
+// bytes written and read (five 16-byte accesses each way), which HBM (used at
+// well under a fifth of its bandwidth by these passes) absorbs.
+// Each pass is one CTA per SM over equal shares of the node warps (see
+// split64.cuh), launched as a programmatic dependent of the one before it.
+// The per-CTA partials (Lambda, E_M, xi) keep the fused kernel's layout.
 #include "split64.cuh"
 #include "tma.cuh"
 
 namespace glemur {
 
-// Boundary nodes enumerated densely, grouped so that the lanes of a warp
-// share one stencil variant per axis: the inner parts of the two z faces,
-// the two y faces and the two x faces (one boundary index coordinate), the
-// edges along x, y and z (two), then the eight corners; b in
-// [0, N - interior).  (A warp mixes variants only where it straddles two
-// groups.)  The host's persistent-kernel plan mirrors this order.
+// Boundary nodes enumerated in groups of one stencil variant each (which
+// axes are one-sided): the inner parts of the two z faces, the two y faces
+// and the two x faces (one boundary index coordinate), the edges along x, y
+// and z (two), then the eight corners.  Every group starts a new warp, so no
+// warp runs more than one variant: a warp with n of them takes its quarter of
+// the SM n times as long, and with the groups packed one warp at their end
+// had four -- 14000 cycles of a 33000-cycle pass B at 64^3, most of it at
+// 16^3.  b in [0, boundary_items); -1 for the idle lanes of a group's last
+// warp.  The host's persistent-kernel plan mirrors this order.
 __device__ __forceinline__ int boundary_node(const SplitArgs& a, int b, int& i, int& j, int& k) {
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const int xi = nx - 2, yi = ny - 2, zi = nz - 2;
   const int fz = xi * yi, fy = xi * zi, fx = yi * zi;
-  if (b < 2 * fz) {
+  bool idle;
+  if (b < pad32(2 * fz)) {
+    idle = b >= 2 * fz;
     k = b < fz ? 0 : nz - 1;
-    const int r = b < fz ? b : b - fz;
-    i = 1 + r % xi;
-    j = 1 + r / xi;
-  } else if ((b -= 2 * fz) < 2 * fy) {
+    const int r = b < fz ? b : b - fz, q = a.dx.div(r);
+    i = 1 + r - q * xi;
+    j = 1 + q;
+  } else if ((b -= pad32(2 * fz)) < pad32(2 * fy)) {
+    idle = b >= 2 * fy;
     j = b < fy ? 0 : ny - 1;
-    const int r = b < fy ? b : b - fy;
-    i = 1 + r % xi;
-    k = 1 + r / xi;
-  } else if ((b -= 2 * fy) < 2 * fx) {
+    const int r = b < fy ? b : b - fy, q = a.dx.div(r);
+    i = 1 + r - q * xi;
+    k = 1 + q;
+  } else if ((b -= pad32(2 * fy)) < pad32(2 * fx)) {
+    idle = b >= 2 * fx;
     i = b < fx ? 0 : nx - 1;
-    const int r = b < fx ? b : b - fx;
-    j = 1 + r % yi;
-    k = 1 + r / yi;
-  } else if ((b -= 2 * fx) < 4 * xi) {
-    const int e = b / xi;
-    i = 1 + b % xi;
+    const int r = b < fx ? b : b - fx, q = a.dy.div(r);
+    j = 1 + r - q * yi;
+    k = 1 + q;
+  } else if ((b -= pad32(2 * fx)) < pad32(4 * xi)) {
+    idle = b >= 4 * xi;
+    const int e = a.dx.div(b);
+    i = 1 + b - e * xi;
     j = (e & 1) ? ny - 1 : 0;
     k = (e & 2) ? nz - 1 : 0;
-  } else if ((b -= 4 * xi) < 4 * yi) {
-    const int e = b / yi;
-    j = 1 + b % yi;
+  } else if ((b -= pad32(4 * xi)) < pad32(4 * yi)) {
+    idle = b >= 4 * yi;
+    const int e = a.dy.div(b);
+    j = 1 + b - e * yi;
     i = (e & 1) ? nx - 1 : 0;
     k = (e & 2) ? nz - 1 : 0;
-  } else if ((b -= 4 * yi) < 4 * zi) {
-    const int e = b / zi;
-    k = 1 + b % zi;
+  } else if ((b -= pad32(4 * yi)) < pad32(4 * zi)) {
+    idle = b >= 4 * zi;
+    const int e = a.dz.div(b);
+    k = 1 + b - e * zi;
     i = (e & 1) ? nx - 1 : 0;
     j = (e & 2) ? ny - 1 : 0;
   } else {
-    b -= 4 * zi;
+    b -= pad32(4 * zi);
+    idle = b >= 8;
     i = (b & 1) ? nx - 1 : 0;
     j = (b & 2) ? ny - 1 : 0;
     k = (b & 4) ? nz - 1 : 0;
   }
-  return (k * ny + j) * nx + i;
+  return idle ? -1 : (k * ny + j) * nx + i;
 }
 
 // One column of G from the stage input y along an axis of node stride
@@ -108,14 +113,26 @@ __device__ __forceinline__ void gcol(const double* __restrict__ y, int N, int n,
   }
 }
 
+// Where interior node t's record for pass C starts: the records of a warp's
+// 32 nodes lie side by side, value by value, so each of a record's five
+// 16-byte accesses is one contiguous 512 bytes for the warp.  FP64 and memory
+// instructions share an issue queue here, and a warp's accesses hold it for
+// every 128-byte line they touch: with the records one after another (80
+// bytes apart) those five touched 100 lines, of 200 in all, in a pass whose
+// FP64 instructions take 864 cycles a node warp (129 x 97 x 75: 1029 -> 1019
+// us an attempt).
+__device__ __forceinline__ double2* node_record(const SplitArgs& a, int t) {
+  return reinterpret_cast<double2*>(a.Gb) + ((size_t)(t >> 5) * 160 + (t & 31));
+}
+
 // det G, 1/det G and B = G B0s / det G at node n from its columns (eq. "B
 // transformation"); B (and 1/det G if rb is set) stored at node nw (n
 // itself, or a periodic ghost node that carries n's B), with G: the
 // differences and 1/det G interleaved for pass C (interior nodes).  Returns
 // the node's energy term zeta |B|^2 det G if `energy`.
 template <bool WITH_G>
-__device__ __forceinline__ double split_B_finish(const SplitArgs& a, int N, int n, int i, int j,
-                                                 int k, bool state, bool energy, int nw,
+__device__ __forceinline__ double split_B_finish(const SplitArgs& a, int N, int n, int t, int i,
+                                                 int j, int k, bool state, bool energy, int nw,
                                                  double g0[3], double g1[3], double g2[3]) {
   g0[0] += a.h2[0];
   g1[1] += a.h2[1];
@@ -125,14 +142,13 @@ __device__ __forceinline__ double split_B_finish(const SplitArgs& a, int N, int 
     atomicOr(&a.st->flags, state ? FLAG_COLLAPSED : FLAG_FOLDED_TRIAL);
   const double r = recip(det);
   if (WITH_G) {
-    // the node's differences and 1/det G for pass C, as five 16-byte
-    // stores (10 N doubles: size_t offsets)
-    double2* q = reinterpret_cast<double2*>(a.Gb + (size_t)n * 10);
+    // the node's differences and 1/det G for pass C
+    double2* q = node_record(a, t);
     q[0] = make_double2(g0[0], g0[1]);
-    q[1] = make_double2(g0[2], g1[0]);
-    q[2] = make_double2(g1[1], g1[2]);
-    q[3] = make_double2(g2[0], g2[1]);
-    q[4] = make_double2(g2[2], r);
+    q[32] = make_double2(g0[2], g1[0]);
+    q[64] = make_double2(g1[1], g1[2]);
+    q[96] = make_double2(g2[0], g2[1]);
+    q[128] = make_double2(g2[2], r);
   }
   const double b0 = __ldg(&a.B0s[n]), b1 = __ldg(&a.B0s[N + n]), b2 = __ldg(&a.B0s[2 * N + n]);
   double B[3];
@@ -153,13 +169,13 @@ __device__ __forceinline__ double split_B_finish(const SplitArgs& a, int N, int 
 template <class LD>
 __device__ __forceinline__ double split_B_interior(const SplitArgs& a,
                                                    const double* __restrict__ y, int N, int n,
-                                                   int i, int j, int k, bool state,
+                                                   int t, int i, int j, int k, bool state,
                                                    bool energy) {
   double g0[3], g1[3], g2[3];
   gcol<false, LD>(y, N, n, 1, 1, g0);
   gcol<false, LD>(y, N, n, a.nx, 1, g1);
   gcol<false, LD>(y, N, n, a.nx * a.ny, 1, g2);
-  return split_B_finish<true>(a, N, n, i, j, k, state, energy, n, g0, g1, g2);
+  return split_B_finish<true>(a, N, n, t, i, j, k, state, energy, n, g0, g1, g2);
 }
 
 // B at a boundary node (or, with periodic z, at the partner of a ghost
@@ -175,7 +191,7 @@ __device__ __forceinline__ double split_B_bvar(const SplitArgs& a, const double*
   gcol<OX, LD>(y, N, n, 1, sx, g0);
   gcol<OY, LD>(y, N, n, a.nx, sy, g1);
   gcol<OZ, LD>(y, N, n, a.nx * a.ny, sz, g2);
-  return split_B_finish<false>(a, N, n, i, j, k, state, energy, nw, g0, g1, g2);
+  return split_B_finish<false>(a, N, n, 0, i, j, k, state, energy, nw, g0, g1, g2);
 }
 
 template <class LD>
@@ -207,22 +223,26 @@ __device__ __forceinline__ double split_B_boundary(const SplitArgs& a,
 template <int S, class LD>
 __device__ __forceinline__ void pass_B(const SplitArgs& a, int cur, double* red) {
   const int N = a.nx * a.ny * a.nz;
-  const int NI = (a.nx - 2) * (a.ny - 2) * (a.nz - 2);
   const double* y = S == 0 ? a.d[cur] : a.ys[S & 1];
   const bool energy = S == 0 && a.diag;
   double eacc = 0.0;
   int tb, te;
-  cta_range(NI, tb, te);
+  cta_range(a.inner_b, tb, te);
 #pragma unroll 2  // two nodes' loads in flight (48 -> 64 registers, +1 % at 64^3)
   for (int t = tb + threadIdx.x; t < te; t += blockDim.x) {
     int i, j, k;
     const int n = interior_node(a, t, i, j, k);
-    eacc += split_B_interior<LD>(a, y, N, n, i, j, k, S == 0, energy);
+    eacc += split_B_interior<LD>(a, y, N, n, t, i, j, k, S == 0, energy);
   }
-  cta_range(N - NI, tb, te);
-  for (int b = tb + threadIdx.x; b < te; b += blockDim.x) {
+  // the boundary nodes take up where the interior ones left off
+  const int nw = blockDim.x >> 5;
+  int wb = (threadIdx.x >> 5) - ((te - tb + 31) >> 5);
+  while (wb < 0) wb += nw;
+  cta_range(a.bound_b, tb, te, gridDim.x - 1 - blockIdx.x);
+  for (int b = tb + 32 * wb + (threadIdx.x & 31); b < te; b += blockDim.x) {
     int i, j, k;
     const int n = boundary_node(a, b, i, j, k);
+    if (n < 0) continue;
     const int sx = i == 0 ? 1 : (i == a.nx - 1 ? -1 : 0);
     const int sy = j == 0 ? 1 : (j == a.ny - 1 ? -1 : 0);
     const int sz = k == 0 ? 1 : (k == a.nz - 1 ? -1 : 0);
@@ -243,17 +263,12 @@ __device__ __forceinline__ void pass_B(const SplitArgs& a, int cur, double* red)
   }
 }
 
-// No minimum-CTA bound: the later stages' pass B fits 64 registers (four
-// CTAs per SM) by itself, the first (with the energy sum) takes 76 (three
-// CTAs, its grid sized to match); forcing four CTAs on every stage made each
-// of them spill.
 template <int S>
-__global__ void __launch_bounds__(256) k_split_B(const SplitArgs a) {
-  pdl_wait();
-  const DevState* st = a.st;
-  if (!a.force && (st->status != ST_OK || st->n_accept >= st->target)) return;
-  __shared__ double red[8];
-  pass_B<S, LdRO>(a, st->cur, red);
+__global__ void __launch_bounds__(DENSE_T, 1) k_split_B(const SplitArgs a) {
+  int cur;
+  if (!dense_start<S == 0>(a, cur)) return;
+  __shared__ double red[32];
+  pass_B<S, LdRO>(a, cur, red);
 }
 
 // One octilateral loop of the next-nearest-neighbour current (section
@@ -369,9 +384,8 @@ __device__ __forceinline__ void nnn_current(const SplitArgs& a, const double* __
 
 // Pass C (stage s): current and velocity at interior nodes; k_s and the
 // next stage input, or (s = 5) the update, the error and k6.  CURL 0: the
-// nearest-neighbour current, held to 64 registers (four CTAs, 32 warps, per
-// SM); CURL 2: the next-nearest-neighbour current (a comparison option,
-// two CTAs per SM).
+// nearest-neighbour current; CURL 2: the next-nearest-neighbour current (a
+// comparison option).
 template <int S, int CURL, class LD>
 __device__ __forceinline__ void pass_C(const SplitArgs& a, int cur, double* red) {
   constexpr bool FINAL = S == 5;
@@ -385,9 +399,8 @@ __device__ __forceinline__ void pass_C(const SplitArgs& a, int cur, double* red)
   for (int j = 0; j < 5; ++j) an[j] = (!FINAL && j <= S) ? LD::ld(&st->dta[S + 1][j]) : 0.0;
   Acc<double> acc;
   const int sy = a.nx, sz = a.nx * a.ny;
-  const int NI = (a.nx - 2) * (a.ny - 2) * (a.nz - 2);
   int tb, te;
-  cta_range(NI, tb, te);
+  cta_range(a.inner_c, tb, te);
   for (int t = tb + threadIdx.x; t < te; t += blockDim.x) {
     int i, j, k;
     const int n = interior_node(a, t, i, j, k);
@@ -396,9 +409,9 @@ __device__ __forceinline__ void pass_C(const SplitArgs& a, int cur, double* red)
       nnn_current<LD>(a, S == 0 ? d : a.ys[S & 1], N, n, J, B);
     } else {
       double g0[3], g1[3], g2[3], P0[3], P1[3], P2[3];
-      const double2* q = reinterpret_cast<const double2*>(a.Gb + (size_t)n * 10);
-      const double2 q0 = LD::ld2(q), q1 = LD::ld2(q + 1), q2 = LD::ld2(q + 2),
-                    q3 = LD::ld2(q + 3), q4 = LD::ld2(q + 4);
+      const double2* q = node_record(a, t);
+      const double2 q0 = LD::ld2(q), q1 = LD::ld2(q + 32), q2 = LD::ld2(q + 64),
+                    q3 = LD::ld2(q + 96), q4 = LD::ld2(q + 128);
       g0[0] = q0.x; g0[1] = q0.y; g0[2] = q1.x;
       g1[0] = q1.y; g1[1] = q2.x; g1[2] = q2.y;
       g2[0] = q3.x; g2[1] = q3.y; g2[2] = q4.x;
@@ -437,20 +450,18 @@ __device__ __forceinline__ void pass_C(const SplitArgs& a, int cur, double* red)
 }
 
 template <int S, int CURL>
-__global__ void __launch_bounds__(256, CURL == 2 ? 2 : 4) k_split_C(const SplitArgs a) {
-  pdl_wait();
-  const DevState* st = a.st;
-  if (!a.force && (st->status != ST_OK || st->n_accept >= st->target)) return;
-  __shared__ double red[8];
-  pass_C<S, CURL, LdRO>(a, st->cur, red);
+__global__ void __launch_bounds__(CURL == 2 ? DENSE_T2 : DENSE_T, 1) k_split_C(const SplitArgs a) {
+  int cur;
+  if (!dense_start<false>(a, cur)) return;
+  __shared__ double red[32];
+  pass_C<S, CURL, LdRO>(a, cur, red);
 }
 
 // ---- persistent attempts ------------------------------------------------
 //
 // One cooperative launch runs whole attempts: the twelve passes and the
 // step control, with no kernel boundary between them.  Each CTA keeps the
-// node ranges it has in the per-pass kernels (the grid is the CTAs the SMs
-// hold, all resident), and instead of a grid-wide boundary after each pass
+// node ranges it has in the per-pass kernels (one CTA per SM, all resident), and instead of a grid-wide boundary after each pass
 // it waits only for the node planes its next pass reads:
 //   pass B of stage s at plane p reads the stage input at planes p-2..p+2,
 //     written by pass C of stage s-1 (the one-sided boundary stencil reaches
@@ -467,9 +478,10 @@ __global__ void __launch_bounds__(256, CURL == 2 ? 2 : 4) k_split_C(const SplitA
 // bounded: after 2 s it raises FLAG_TIMEOUT and status TIMEOUT and the CTA
 // leaves; the others see the flag in their own waits and leave too.
 // Results are bit-identical to the per-pass kernels: each node's
-// arithmetic is the same.  Measured on GB300 it is about 5 % slower than
-// the per-pass kernels chained by programmatic dependent launch (64^3 and
-// 96^3 braids), so it runs only on request (GLEMUR_PERSIST=1).
+// arithmetic is the same.  Measured on GB300 it is slower than the per-pass
+// kernels chained by programmatic dependent launch (16^3: 76 against 56 us an
+// attempt, 64^3: 344 against 302), so it runs only on request
+// (GLEMUR_PERSIST=1).
 
 constexpr unsigned long long PERSIST_WAIT_NS = 2000000000ull;
 
@@ -545,9 +557,9 @@ __device__ __forceinline__ void persist_publish(const int* iv, int nint, int* cn
 }
 
 template <int CURL>
-__global__ void __launch_bounds__(256, CURL == 2 ? 2 : 4)
+__global__ void __launch_bounds__(CURL == 2 ? DENSE_T2 : DENSE_T, 1)
     k_attempts_persist(const SplitArgs a, const PersistArgs pa) {
-  __shared__ double red[8];
+  __shared__ double red[32];
   __shared__ double sh[96];
   __shared__ int ok, last;
   DevState* st = a.st;
@@ -591,7 +603,7 @@ __global__ void __launch_bounds__(256, CURL == 2 ? 2 : 4)
     __syncthreads();
     if (last) {
       __threadfence();
-      control_block<LdCoherent>(st, a.part, a.nblocks, a.diag, pa.dtlog, sh);
+      control_block<LdCoherent>(st, a.part, a.nblocks, a.diag, pa.dtlog, sh, [] {});
       __syncthreads();
       if (threadIdx.x == 0) {
         __threadfence();
@@ -620,22 +632,13 @@ __global__ void __launch_bounds__(256, CURL == 2 ? 2 : 4)
   }
 }
 
-// CTAs of 256 threads per SM the persistent kernel can hold, and its launch
-// (cooperative: every CTA resident, or the launch fails).
-int persist_ctas_per_sm(int curl) {
-  int n = 0;
-  if (curl == 2)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_attempts_persist<2>, 256, 0);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_attempts_persist<0>, 256, 0);
-  return n;
-}
-
+// The persistent kernel's launch (cooperative: every CTA resident, or the
+// launch fails).
 cudaError_t launch_f64_persist(const SplitArgs& a, const PersistArgs& pa, int grid, int curl,
                                cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(a.threads_b);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -647,37 +650,31 @@ cudaError_t launch_f64_persist(const SplitArgs& a, const PersistArgs& pa, int gr
   return cudaLaunchKernelEx(&cfg, k_attempts_persist<0>, a, pa);
 }
 
-// CTAs of 256 threads per SM that pass B and pass C of each stage can hold
-// (pass C with the current `curl`: 0 nearest, 2 next-nearest neighbours).
-void split_ctas_per_sm(int b[6], int c[6], int curl) {
-  void (*kb[6])(const SplitArgs) = {k_split_B<0>, k_split_B<1>, k_split_B<2>,
-                                    k_split_B<3>, k_split_B<4>, k_split_B<5>};
-  void (*kc0[6])(const SplitArgs) = {k_split_C<0, 0>, k_split_C<1, 0>, k_split_C<2, 0>,
-                                     k_split_C<3, 0>, k_split_C<4, 0>, k_split_C<5, 0>};
-  void (*kc2[6])(const SplitArgs) = {k_split_C<0, 2>, k_split_C<1, 2>, k_split_C<2, 2>,
-                                     k_split_C<3, 2>, k_split_C<4, 2>, k_split_C<5, 2>};
-  void (**kc)(const SplitArgs) = curl == 2 ? kc2 : kc0;
-  for (int s = 0; s < 6; ++s) {
-    b[s] = c[s] = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b[s], kb[s], 256, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c[s], kc[s], 256, 0);
-    if (b[s] < 1) b[s] = 1;
-    if (c[s] < 1) c[s] = 1;
-  }
+// Let the passes ask for DENSE_SMEM.
+cudaError_t prepare_f64_split() {
+  void (*k[18])(const SplitArgs) = {
+      k_split_B<0>,    k_split_B<1>,    k_split_B<2>,    k_split_B<3>,    k_split_B<4>,
+      k_split_B<5>,    k_split_C<0, 0>, k_split_C<1, 0>, k_split_C<2, 0>, k_split_C<3, 0>,
+      k_split_C<4, 0>, k_split_C<5, 0>, k_split_C<0, 2>, k_split_C<1, 2>, k_split_C<2, 2>,
+      k_split_C<3, 2>, k_split_C<4, 2>, k_split_C<5, 2>};
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < 18 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(k[i], cudaFuncAttributeMaxDynamicSharedMemorySize, DENSE_SMEM);
+  return e;
 }
 
-// Launch both passes of stage s (grid_b[s], grid_c[s] CTAs of 256 threads)
+// Launch both passes of stage s
 // with the current `curl` (0 nearest, 2 next-nearest neighbours).
 cudaError_t launch_f64_split(const SplitArgs& a, int stage, cudaStream_t s, int curl) {
   if (stage < 0 || stage > 5 || (curl != 0 && curl != 2)) return cudaErrorInvalidValue;
-  const dim3 gb(a.grid_b[stage]), gc(a.grid_c[stage]);
+  const dim3 gb(a.grid_b), gc(a.grid_c), tb(a.threads_b), tc(a.threads_c);
   cudaError_t e = cudaSuccess;
 #define GLEMUR_SPLIT_CASE(SS)                                                          \
   case SS:                                                                             \
-    e = launch_pdl(k_split_B<SS>, gb, dim3(256), 0, s, a);                             \
+    e = launch_pdl(k_split_B<SS>, gb, tb, DENSE_SMEM, s, a);                             \
     if (e == cudaSuccess)                                                              \
-      e = curl == 2 ? launch_pdl(k_split_C<SS, 2>, gc, dim3(256), 0, s, a)             \
-                    : launch_pdl(k_split_C<SS, 0>, gc, dim3(256), 0, s, a);            \
+      e = curl == 2 ? launch_pdl(k_split_C<SS, 2>, gc, tc, DENSE_SMEM, s, a)             \
+                    : launch_pdl(k_split_C<SS, 0>, gc, tc, DENSE_SMEM, s, a);            \
     break;
   switch (stage) {
     GLEMUR_SPLIT_CASE(0)

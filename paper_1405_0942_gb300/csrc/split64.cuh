@@ -41,25 +41,50 @@ struct LdL2 {
   }
 };
 
-// This CTA's node range: warps [W b / G, W (b+1) / G) of the W = N/32 node
-// warps (rounded up), as node indices [begin, end).
-__device__ __forceinline__ void cta_range(int N, int& begin, int& end) {
-  const long long W = (N + 31) / 32;
-  const long long w0 = W * blockIdx.x / gridDim.x, w1 = W * (blockIdx.x + 1) / gridDim.x;
-  begin = (int)(w0 * 32);
-  end = (int)(w1 * 32 < N ? w1 * 32 : N);
+// How the dense passes are spread.  The FP64 pipe belongs to an SM's
+// quarter: it takes a warp instruction every 64 cycles, and a single warp
+// keeps it 97 % busy (a dependent DFMA takes 67).  So what counts is that
+// every quarter gets the same number of node warps.  A pass runs one CTA per
+// SM, each over an equal range of whole warps of nodes, and the CTA's warps
+// (a multiple of four, warp w on quarter w mod 4) take the range's node warps
+// in turn, so the quarters of an SM differ by one at most.  (Four CTAs of
+// eight warps per SM, each with twelve node warps, gave the first quarter 16
+// where the mean is 12.25: 64^3.)  Small grids get no more warps per CTA than
+// an SM's share, four at least, so that one node warp has a quarter to
+// itself.  Together with the variant groups of boundary_node, index division
+// by multiplication and no 64-bit division, an attempt went from 95 to 56 us
+// at 16^3, 106 to 74 at 33^3, 211 to 155 at 48^3 and 349 to 302 at 64^3.
+//
+// CTA b's range [begin, end) of the nodes w shares out.  (Pass B takes the
+// boundary's in reverse, so that one CTA does not get both extra warps.)
+__device__ __forceinline__ void cta_range(const WarpShare& w, int& begin, int& end,
+                                          int b = blockIdx.x) {
+  begin = 32 * (b * w.each + min(b, w.extra));
+  end = min(begin + 32 * (w.each + (b < w.extra)), w.n);
 }
 
 // Interior nodes enumerated densely: t in [0, (nx-2)(ny-2)(nz-2)) -> node.
 // A warp then holds 32 interior nodes, so the interior code (central
 // differences only) runs with no boundary lanes in it.
 __device__ __forceinline__ int interior_node(const SplitArgs& a, int t, int& i, int& j, int& k) {
-  const int nxi = a.nx - 2, nyi = a.ny - 2;
-  i = 1 + t % nxi;
-  const int r = t / nxi;
-  j = 1 + r % nyi;
-  k = 1 + r / nyi;
+  const int r = a.dx.div(t), q = a.dy.div(r);
+  i = 1 + t - r * a.dx.d;
+  j = 1 + r - q * a.dy.d;
+  k = 1 + q;
   return (k * a.ny + j) * a.nx + i;
+}
+
+// The start of a dense pass: false if stepping has stopped.  FIRST: the
+// first kernel of an attempt, which waits before it reads anything; the
+// others read the control state ahead of the wait (see launch_pdl).
+template <bool FIRST>
+__device__ __forceinline__ bool dense_start(const SplitArgs& a, int& cur) {
+  if (FIRST) pdl_wait();
+  const DevState* st = a.st;
+  const bool stop = !a.force && (st->status != ST_OK || st->n_accept >= st->target);
+  cur = st->cur;
+  if (!FIRST) pdl_wait();
+  return !stop;
 }
 
 // This CTA's partial of kind `kind`; the slots of the partial stride beyond
