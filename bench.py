@@ -56,20 +56,21 @@ MIN_TIMED_S = 1.0              # repeat the block of timed attempts until this
 # captured from (kernel_source_hash()); a workload without an entry, or one
 # whose kernels have changed since, reports null
 NCU_TRAFFIC = {
-    ("braid64", "fp64", "mimetic"): (57730944, "633176018912"),
-    ("braid64", "fp64", "direct"): (31326890, "633176018912"),
-    ("braid64", "fp64", "nnn"): (44000170, "633176018912"),
-    ("periodic64", "fp64", "mimetic"): (57533269, "633176018912"),
-    ("braid64", "mixed", "mimetic"): (15672021, "633176018912"),
-    ("braid64", "mixed", "direct"): (15827456, "633176018912"),
-    ("braid128", "mixed", "mimetic"): (152441216, "633176018912"),
-    ("prod384", "mixed", "mimetic"): (4717954389, "633176018912"),
+    ("braid64", "fp64", "mimetic"): (57730944, "fdb4557c2692"),
+    ("braid64", "fp64", "direct"): (31326890, "fdb4557c2692"),
+    ("braid64", "fp64", "nnn"): (44000170, "fdb4557c2692"),
+    ("periodic64", "fp64", "mimetic"): (57533269, "fdb4557c2692"),
+    ("braid64", "mixed", "mimetic"): (15672021, "fdb4557c2692"),
+    ("braid64", "mixed", "direct"): (15827456, "fdb4557c2692"),
+    ("braid128", "mixed", "mimetic"): (152441216, "fdb4557c2692"),
+    ("prod384", "mixed", "mimetic"): (4717954389, "fdb4557c2692"),
 }
 
 
 # sources the stage kernels and their launches are built from (the adjoint,
 # the diagnostics and the allocation-free energy are not on the timed path)
-STAGE_SOURCES_EXCLUDED = ("adjoint.cu", "diagnostics.cu", "energy_static.cu")
+STAGE_SOURCES_EXCLUDED = ("adjoint.cu", "diagnostics.cu", "energy_static.cu", "kern_f64_vjp.cu",
+                          "vjp64.cuh")
 
 
 def kernel_source_hash():

@@ -32,6 +32,7 @@
 
 #include "glemur.h"
 #include "glemur_dev.cuh"
+#include "vjp64.cuh"
 
 namespace glemur {
 
@@ -642,8 +643,9 @@ __global__ void k_param_contract(long long M, const double* dB, const double* mu
 namespace glemur {
 // Provided by glemur.cu.
 int ctx_recompute_stages(glemur_ctx* c, double dt, void* k6);
-int ctx_recompute_stages_saved(glemur_ctx* c, double dt, void* k6, double* const* yS,
-                               double* const* BS, double* const* RS);
+int ctx_recompute_stages_saved(glemur_ctx* c, double dt, double* const* yS, double* const* BS,
+                               double* const* GS);
+void ctx_dense_grid(const glemur_ctx* c, int most, int* grid, int* threads);
 int ctx_info(glemur_ctx* c, int* nx, int* ny, int* nz, double h[3], int* precision,
              void** d_cur, void** B0s, void** k, void** stream);
 }  // namespace glemur
@@ -660,7 +662,7 @@ size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 // xi partials and two small pointer tables.
 struct AdjLayout {
   size_t k6, y, Bb, rb, lamk, lamy, lamP, lamg, lamr, lamB, lamB2, lamu, mu, pv, pi, ptr,
-      yS, BS, RS, total, fstride, rstride;
+      yS, BS, GS, total, fstride, gstride;
 };
 
 constexpr int kXiBlocks = 1024;
@@ -687,13 +689,14 @@ AdjLayout adj_layout(int nx, int ny, int nz, int precision) {
   L.pv = o; o += al(kXiBlocks * 8 + 8);
   L.pi = o; o += al(kXiBlocks * 4);
   L.ptr = o; o += 256;
-  // FP64: every stage's input (y_1..y_5), B and 1/det G, kept by the
-  // forward recompute so the reverse loop need not form them again
-  L.rstride = al(N * 8);
+  // FP64: every stage's input (y_1..y_5), B and node records (G and 1/det G,
+  // whole warps of interior nodes), kept by the forward recompute so the
+  // reverse loop need not form them again
+  L.gstride = al(10 * (N + 31) * 8);
   if (precision == GLEMUR_FP64) {
     L.yS = o; o += 5 * L.fstride;
     L.BS = o; o += 6 * L.fstride;
-    L.RS = o; o += 6 * L.rstride;
+    L.GS = o; o += 6 * L.gstride;
   }
   L.total = o;
   return L;
@@ -738,14 +741,26 @@ int nblk(long long n) {
   return (int)(b < 8192 ? (b < 1 ? 1 : b) : 8192);
 }
 
+// The same table on the host.
+const double kA[6][6] = {
+    {0, 0, 0, 0, 0, 0},
+    {1.0 / 5.0, 0, 0, 0, 0, 0},
+    {3.0 / 40.0, 9.0 / 40.0, 0, 0, 0, 0},
+    {3.0 / 10.0, -9.0 / 10.0, 6.0 / 5.0, 0, 0, 0},
+    {-11.0 / 54.0, 5.0 / 2.0, -70.0 / 27.0, 35.0 / 27.0, 0, 0},
+    {1631.0 / 55296.0, 175.0 / 512.0, 575.0 / 13824.0, 44275.0 / 110592.0, 253.0 / 4096.0,
+     0}};
+const double kB5[6] = {37.0 / 378.0, 0.0, 250.0 / 621.0, 125.0 / 594.0, 0.0, 512.0 / 1771.0};
+
 // Five stage-input buffers (pointers by value).
 struct YSave {
   double* p[5];
 };
 
 // Boundary entries of the saved stage inputs y_1..y_5: the fixed boundary
-// positions (the forward passes write interior nodes only).
-__global__ void k_adj_seed_boundary(AdjGeom g, const double* d, YSave ys) {
+// positions (the forward passes write interior nodes only); and of the
+// adjoints of P, zero: no difference is taken there.
+__global__ void k_adj_seed_boundary(AdjGeom g, const double* d, YSave ys, double* lamP) {
   pdl_wait();
   pdl_trigger();
   const int N = g.nx * g.ny * g.nz, NI = (g.nx - 2) * (g.ny - 2) * (g.nz - 2);
@@ -756,7 +771,62 @@ __global__ void k_adj_seed_boundary(AdjGeom g, const double* d, YSave ys) {
       const double v = d[c * N + n];
       for (int q = 0; q < 5; ++q) ys.p[q][c * N + n] = v;
     }
+    for (int q = 0; q < 9; ++q) lamP[q * N + n] = 0.0;
   }
+}
+
+// The reverse step of an FP64 two-pass context, from the recompute's saved
+// data (kern_f64_vjp.cu).  BADARG for other contexts, with nothing done.
+int vjp_step_saved(glemur_ctx* c, const Adj& A, double dt, const double* lam_next, double* lam,
+                   double* mu_B0) {
+  double *yS[6] = {nullptr}, *BS[6], *GS[6];
+  YSave ysave;
+  for (int q = 1; q < 6; ++q) ysave.p[q - 1] = yS[q] = A.P(A.L.yS + (q - 1) * A.L.fstride);
+  for (int q = 0; q < 6; ++q) {
+    BS[q] = A.P(A.L.BS + q * A.L.fstride);
+    GS[q] = A.P(A.L.GS + q * A.L.gstride);
+  }
+  launch_pdl(k_adj_seed_boundary, dim3(nblk(A.N)), dim3(256), 0, A.s, A.g, (const double*)A.d,
+             ysave, A.P(A.L.lamP));
+  const int rc = ctx_recompute_stages_saved(c, dt, yS, BS, GS);
+  if (rc) return rc;
+  VjpArgs v;
+  v.nx = A.g.nx;
+  v.ny = A.g.ny;
+  v.nz = A.g.nz;
+  for (int a = 0; a < 3; ++a) {
+    v.h2[a] = A.g.h2[a];
+    v.s[a] = A.g.s[a];
+  }
+  v.B0s = (const double*)A.B0s;
+  v.lam_next = lam_next;
+  for (int j = 0; j < 6; ++j) v.ly[j] = A.P(A.L.lamk + j * A.L.fstride);
+  v.lamP = A.P(A.L.lamP);
+  v.lamg = A.P(A.L.lamg);
+  v.lamr = A.P(A.L.lamr);
+  v.lamB = A.P(A.L.lamB);
+  v.lam = lam;
+  v.mu_B0 = mu_B0;
+  ctx_dense_grid(c, DENSE_T2, &v.grid, &v.threads);
+  const long long xi = v.nx - 2, yi = v.ny - 2, zi = v.nz - 2;
+  v.inner = warp_share(xi * yi * zi, v.grid);
+  v.faces = warp_share((long long)pad32((int)(2 * xi * yi)) + pad32((int)(2 * xi * zi)) +
+                           pad32((int)(2 * yi * zi)), v.grid);
+  v.bound = warp_share(boundary_items(v.nx, v.ny, v.nz), v.grid);
+  v.dx = fast_div((int)xi);
+  v.dy = fast_div((int)yi);
+  v.dz = fast_div((int)zi);
+  for (int s = 5; s >= 0; --s) {
+    v.y = s == 0 ? (const double*)A.d : yS[s];
+    v.Bb = BS[s];
+    v.rec = GS[s];
+    v.cb = dt * kB5[s];
+    for (int j = 0; j < 6; ++j) v.ca[j] = j > s ? dt * kA[j][s] : 0.0;
+    v.ly_out = (double*)v.ly[s];
+    const cudaError_t e = launch_f64_vjp(v, s, A.s);
+    if (e != cudaSuccess) return GLEMUR_ERR_CUDA;
+  }
+  return cudaStreamSynchronize(A.s) == cudaSuccess ? GLEMUR_OK : GLEMUR_ERR_CUDA;
 }
 
 // The stage VJP at the stage input y (B and 1/det G in Bb, rb; formed here
@@ -791,26 +861,11 @@ template <typename T>
 int vjp_step_t(glemur_ctx* c, const Adj& A, double dt, const double* lam_next, double* lam,
                double* mu_B0) {
   const int N3 = 3 * A.N;
-  // FP64 two-pass contexts: the recompute keeps every stage's input, B and
-  // 1/det G; otherwise the reverse loop forms them again
-  double* yS[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  double* BS[6];
-  double* RS[6];
-  bool saved = false;
   if (A.precision == GLEMUR_FP64) {
-    YSave ysave;
-    for (int q = 1; q < 6; ++q) ysave.p[q - 1] = yS[q] = A.P(A.L.yS + (q - 1) * A.L.fstride);
-    for (int q = 0; q < 6; ++q) {
-      BS[q] = A.P(A.L.BS + q * A.L.fstride);
-      RS[q] = A.P(A.L.RS + q * A.L.rstride);
-    }
-    launch_pdl(k_adj_seed_boundary, dim3(nblk(A.N)), dim3(256), 0, A.s, A.g, (const double*)A.d,
-               ysave);
-    const int rs = ctx_recompute_stages_saved(c, dt, A.ws + A.L.k6, yS, BS, RS);
-    if (rs != GLEMUR_OK && rs != GLEMUR_ERR_BADARG) return rs;
-    saved = rs == GLEMUR_OK;
+    const int rs = vjp_step_saved(c, A, dt, lam_next, lam, mu_B0);
+    if (rs != GLEMUR_ERR_BADARG) return rs;
   }
-  int rc = saved ? GLEMUR_OK : ctx_recompute_stages(c, dt, A.ws + A.L.k6);
+  const int rc = ctx_recompute_stages(c, dt, A.ws + A.L.k6);
   if (rc) return rc;
   double* lamk_h[6];
   for (int j = 0; j < 6; ++j) lamk_h[j] = A.P(A.L.lamk + j * A.L.fstride);
@@ -824,15 +879,10 @@ int vjp_step_t(glemur_ctx* c, const Adj& A, double dt, const double* lam_next, d
   launch_pdl(k_adj_zero, dim3(nblk(N3)), dim3(256), 0, A.s, N3, A.P(A.L.mu));
   launch_pdl(k_adj_seed, dim3(nblk(N3)), dim3(256), 0, A.s, N3, lam_next, dt, lam, lamk_d);
   for (int s = 5; s >= 0; --s) {
-    if (saved) {
-      stage_vjp<T>(A, s == 0 ? (const double*)A.d : yS[s], BS[s], RS[s], false, lamk_h[s],
-                   nullptr, 0.0, s, dt, lam, lamk_d);
-    } else {
-      launch_pdl(k_adj_stage_input<T>, dim3(nblk(N3)), dim3(256), 0, A.s, N3, (const T*)A.d, kp_d,
-                 s, dt, A.P(A.L.y));
-      stage_vjp<T>(A, A.P(A.L.y), A.P(A.L.Bb), A.P(A.L.rb), true, lamk_h[s], nullptr, 0.0, s,
-                   dt, lam, lamk_d);
-    }
+    launch_pdl(k_adj_stage_input<T>, dim3(nblk(N3)), dim3(256), 0, A.s, N3, (const T*)A.d, kp_d,
+               s, dt, A.P(A.L.y));
+    stage_vjp<T>(A, A.P(A.L.y), A.P(A.L.Bb), A.P(A.L.rb), true, lamk_h[s], nullptr, 0.0, s, dt,
+                 lam, lamk_d);
   }
   launch_pdl(k_adj_mu_out, dim3(nblk(A.N)), dim3(256), 0, A.s, A.g, A.P(A.L.mu), mu_B0);
   e = cudaGetLastError();

@@ -15,6 +15,7 @@
 #include "glemur.h"
 #include "glemur_dev.cuh"
 #include "tma.cuh"
+#include "vjp64.cuh"
 
 namespace glemur {
 cudaError_t launch_f64_mimetic(const StageArgs<double>& a, int stage, dim3 grid, cudaStream_t s);
@@ -31,7 +32,8 @@ int tile_rows_f32_mimetic();
 int tile_cols_f32_mimetic();
 int ctas_per_sm_f32_direct();
 
-cudaError_t launch_f64_split(const SplitArgs& a, int stage, cudaStream_t s, int curl);
+cudaError_t launch_f64_split(const SplitArgs& a, int stage, cudaStream_t s, int curl,
+                             bool pass_c = true);
 cudaError_t prepare_f64_split();
 cudaError_t prepare_f64_direct();
 cudaError_t launch_f64_persist(const SplitArgs& a, const PersistArgs& pa, int grid, int curl,
@@ -517,7 +519,6 @@ SplitArgs split_args(const glemur_ctx* c, int diag, int force) {
   a.ys[0] = (double*)c->ys[0];
   a.ys[1] = (double*)c->ys[1];
   a.Bb = c->Bb;
-  a.rb = nullptr;  // pass C reads 1/det G with the differences in Gb
   a.Gb = c->Gb;
   a.diag = diag;
   a.force = force;
@@ -783,28 +784,35 @@ int ctx_recompute_stages(glemur_ctx* c, double dt, void* k6) {
 }
 
 // The same recompute for FP64 two-pass contexts, keeping every stage's
-// data for the adjoint: stage s writes B and 1/det G into BS[s], RS[s]
-// (3N and N doubles) and its next input y_{s+1} into yS[s+1] (3N doubles;
+// data for the adjoint: stage s writes B into BS[s] (3N doubles) and its node
+// records into GS[s], and its next input y_{s+1} into yS[s+1] (3N doubles;
 // the caller has put the boundary positions in yS[1..5]); y_0 is the state
-// itself.  BADARG for other contexts (the caller then recomputes stage data
-// itself).
-int ctx_recompute_stages_saved(glemur_ctx* c, double dt, void* k6, double* const* yS,
-                               double* const* BS, double* const* RS) {
+// itself.  The last stage needs no velocity: its pass C is left out.  BADARG
+// for other contexts (the caller then recomputes stage data itself).
+int ctx_recompute_stages_saved(glemur_ctx* c, double dt, double* const* yS, double* const* BS,
+                               double* const* GS) {
   if (c->o.curl != GLEMUR_CURL_MIMETIC || !c->split) return GLEMUR_ERR_BADARG;
   c->target_unbounded = 0;
   k_set_dt<<<1, 1, 0, c->s>>>(c->st, dt, 0);
   cudaError_t e = cudaGetLastError();
   for (int s = 0; s < 6 && e == cudaSuccess; ++s) {
     SplitArgs a = split_args(c, 0, 1);  // not periodic: the adjoint refuses those
-    a.k[5] = s == 5 ? (double*)k6 : nullptr;
     a.ys[0] = a.ys[1] = nullptr;
     if (s >= 1) a.ys[s & 1] = yS[s];
     if (s < 5) a.ys[(s + 1) & 1] = yS[s + 1];
     a.Bb = BS[s];
-    a.rb = RS[s];
-    e = launch_f64_split(a, s, c->s, 0);
+    a.Gb = GS[s];
+    e = launch_f64_split(a, s, c->s, 0, s < 5);
   }
   return cuda_rc(e);
+}
+
+// Grid of a dense FP64 pass over interior and boundary nodes for this
+// context's device.
+void ctx_dense_grid(const glemur_ctx* c, int most, int* grid, int* threads) {
+  const DenseShape d = dense_shape(c, true, most);
+  *grid = d.grid;
+  *threads = d.threads;
 }
 
 // Geometry, storage and the current accepted displacement (synchronises).
@@ -945,6 +953,7 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   if (e == cudaSuccess) e = mixed ? prepare_f32_mimetic() : prepare_f64_mimetic();
   if (e == cudaSuccess && !mixed) e = prepare_f64_split();
   if (e == cudaSuccess && !mixed) e = prepare_f64_direct();
+  if (e == cudaSuccess && !mixed) e = prepare_f64_vjp();
   c->tma = 0;
   // GLEMUR_TEST_TMA_TIMEOUT=1 (2) makes the TMA prologue wait (the first
   // wait inside the plane loop) also wait on a barrier that never completes,

@@ -179,7 +179,6 @@ struct SplitArgs {
   double* ys[2];       // stage inputs: y_s in ys[s & 1] (s >= 1), 3N each;
                        // boundary entries hold the fixed boundary positions
   double* Bb;          // B, 3N
-  double* rb;          // 1/det G, N, or null (then written to Gb only)
   double* Gb;          // per interior node 10 doubles: g_0, g_1, g_2
                        // (index-space differences, 3 components each) and
                        // 1/det G -- written by pass B, read by pass C

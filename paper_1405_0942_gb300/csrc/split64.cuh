@@ -66,12 +66,97 @@ __device__ __forceinline__ void cta_range(const WarpShare& w, int& begin, int& e
 // Interior nodes enumerated densely: t in [0, (nx-2)(ny-2)(nz-2)) -> node.
 // A warp then holds 32 interior nodes, so the interior code (central
 // differences only) runs with no boundary lanes in it.
-__device__ __forceinline__ int interior_node(const SplitArgs& a, int t, int& i, int& j, int& k) {
+template <class Args>
+__device__ __forceinline__ int interior_node(const Args& a, int t, int& i, int& j, int& k) {
   const int r = a.dx.div(t), q = a.dy.div(r);
   i = 1 + t - r * a.dx.d;
   j = 1 + r - q * a.dy.d;
   k = 1 + q;
   return (k * a.ny + j) * a.nx + i;
+}
+
+// Boundary nodes enumerated in groups of one stencil variant each (which
+// axes are one-sided): the inner parts of the two z faces, the two y faces
+// and the two x faces (one boundary index coordinate), the edges along x, y
+// and z (two), then the eight corners.  Every group starts a new warp, so no
+// warp runs more than one variant: a warp with n of them takes its quarter of
+// the SM n times as long, and with the groups packed one warp at their end
+// had four -- 14000 cycles of a 33000-cycle pass B at 64^3, most of it at
+// 16^3.  b in [0, boundary_items); -1 for the idle lanes of a group's last
+// warp.  The host's persistent-kernel plan mirrors this order.
+template <class Args>
+__device__ __forceinline__ int boundary_node(const Args& a, int b, int& i, int& j, int& k) {
+  const int nx = a.nx, ny = a.ny, nz = a.nz;
+  const int xi = nx - 2, yi = ny - 2, zi = nz - 2;
+  const int fz = xi * yi, fy = xi * zi, fx = yi * zi;
+  bool idle;
+  if (b < pad32(2 * fz)) {
+    idle = b >= 2 * fz;
+    k = b < fz ? 0 : nz - 1;
+    const int r = b < fz ? b : b - fz, q = a.dx.div(r);
+    i = 1 + r - q * xi;
+    j = 1 + q;
+  } else if ((b -= pad32(2 * fz)) < pad32(2 * fy)) {
+    idle = b >= 2 * fy;
+    j = b < fy ? 0 : ny - 1;
+    const int r = b < fy ? b : b - fy, q = a.dx.div(r);
+    i = 1 + r - q * xi;
+    k = 1 + q;
+  } else if ((b -= pad32(2 * fy)) < pad32(2 * fx)) {
+    idle = b >= 2 * fx;
+    i = b < fx ? 0 : nx - 1;
+    const int r = b < fx ? b : b - fx, q = a.dy.div(r);
+    j = 1 + r - q * yi;
+    k = 1 + q;
+  } else if ((b -= pad32(2 * fx)) < pad32(4 * xi)) {
+    idle = b >= 4 * xi;
+    const int e = a.dx.div(b);
+    i = 1 + b - e * xi;
+    j = (e & 1) ? ny - 1 : 0;
+    k = (e & 2) ? nz - 1 : 0;
+  } else if ((b -= pad32(4 * xi)) < pad32(4 * yi)) {
+    idle = b >= 4 * yi;
+    const int e = a.dy.div(b);
+    j = 1 + b - e * yi;
+    i = (e & 1) ? nx - 1 : 0;
+    k = (e & 2) ? nz - 1 : 0;
+  } else if ((b -= pad32(4 * yi)) < pad32(4 * zi)) {
+    idle = b >= 4 * zi;
+    const int e = a.dz.div(b);
+    k = 1 + b - e * zi;
+    i = (e & 1) ? nx - 1 : 0;
+    j = (e & 2) ? ny - 1 : 0;
+  } else {
+    b -= pad32(4 * zi);
+    idle = b >= 8;
+    i = (b & 1) ? nx - 1 : 0;
+    j = (b & 2) ? ny - 1 : 0;
+    k = (b & 4) ? nz - 1 : 0;
+  }
+  return idle ? -1 : (k * ny + j) * nx + i;
+}
+
+// One column of G from the stage input y along an axis of node stride
+// `stride`, without the 2 h_a e_a term.  ONE = false: the central
+// difference v(n+s) - v(n-s).  ONE = true: the second-order one-sided
+// difference into the domain, (4 v(n+s) - 3 v(n)) - v(n+2s) at the low face
+// (sg = +1) and (3 v(n) - 4 v(n-s)) + v(n-2s) at the high face (sg = -1),
+// both as sg times the first form with s -> sg s: the signs ride on
+// constants chosen by a select (multiplying by -1 is exact), so both faces
+// run the same three FP64 instructions per component.
+template <bool ONE, class LD>
+__device__ __forceinline__ void gcol(const double* __restrict__ y, int N, int n, int stride,
+                                     int sg, double out[3]) {
+  const int s = sg * stride;
+  const double c4 = sg > 0 ? 4.0 : -4.0, m3 = sg > 0 ? -3.0 : 3.0, m1 = sg > 0 ? -1.0 : 1.0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double* v = y + c * N;
+    if (!ONE)
+      out[c] = LD::ld(&v[n + stride]) - LD::ld(&v[n - stride]);
+    else
+      out[c] = fma(m1, LD::ld(&v[n + 2 * s]), fma(c4, LD::ld(&v[n + s]), m3 * LD::ld(&v[n])));
+  }
 }
 
 // The start of a dense pass: false if stepping has stopped.  FIRST: the
