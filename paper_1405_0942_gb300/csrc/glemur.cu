@@ -426,28 +426,44 @@ int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe) {
   return best;
 }
 
-// Planes per CTA along z of the mixed mimetic stage.  A CTA of kz planes runs
-// kz + 2 iterations and its prologue takes about half of one.  While all
-// CTAs are resident the time is that of the SM with the most: an iteration
-// takes 0.73 as long alone on an SM as beside a second CTA (128^3: kz = 15,
-// two CTAs per SM, 255 us an attempt; kz = 32, one, 386 us before the barrier
-// was split, 277 us beside it).  Beyond one wave CTAs start as others end and
-// the last ones leave about half a wave idle (128^3: kz = 8, 13 with 1.7,
-// 1.05 waves 291, 325 us).  Long marches lose to short ones on grids of many
-// waves (384^3: kz = 28, 36, 48 take 4.89, 4.85, 4.91 ms, 192 takes 9 % more
-// than 32), hence the limit of 40.
+// Planes per CTA along z of the mixed mimetic stage: the shortest schedule
+// of its CTAs on the SMs' slots.  A CTA of kz planes runs kz + 2 iterations
+// and its prologue takes about half of one; the last slab's CTAs, of the
+// remaining planes, are shorter (one halo plane less) and start last.  They
+// run in the slots the full ones leave free, several in turn where they are
+// short, so a grid of a little more than one wave is often the best: 128^3,
+// kz = 14, 15 (320, 288 CTAs for 304 slots) 243, 255 us an attempt; 101 x 90
+// x 75, kz = 6, 7: 159, 174; 150 x 140 x 130, kz = 24, 26: 498, 530.  With one
+// CTA per SM at most an iteration takes 0.73 as long as with two (64^3, kz =
+// 4, 2: 76, 70 us).  Long marches lose to short ones on grids of many waves
+// (384^3: kz = 28, 36, 48 take 4.89, 4.85, 4.91 ms, 192 takes 9 % more than
+// 32), hence the limit of 40.
 int choose_kz_march(int nz, int gxy, int nsm, int per_sm) {
   const char* env = getenv("GLEMUR_KZ");
   if (env && atoi(env) > 0) return atoi(env) < nz ? atoi(env) : nz;
   if (nsm < 1) nsm = 1;
   if (per_sm < 1) per_sm = 1;
+  const long long slots = (long long)nsm * per_sm;
   int best = nz;
   double best_cost = 1e300;
   for (int kz = 1; kz <= nz && kz <= 40; ++kz) {
-    const long long ctas = (long long)gxy * ((nz + kz - 1) / kz);
-    const double waves = (double)ctas / ((double)nsm * per_sm);
-    const double load = ctas <= nsm ? 0.73 : (waves <= 1.0 ? 1.0 : waves + 0.5);
-    const double cost = load * (kz + 2.5);
+    const long long slabs = (nz + kz - 1) / kz;
+    const long long full = gxy * (slabs - 1), waves = full / slots, left = full % slots;
+    const double tf = kz + 2.5, ts = (double)(nz - (slabs - 1) * kz) + 1.5;
+    // the last wave of full CTAs, and the short ones in its free slots while
+    // it lasts, then in all of them
+    const long long room = slots - left;
+    const double last = left > 0 ? tf : 0.0;
+    const long long turns = left > 0 ? (long long)((tf - 0.01) / ts) + 1 : gxy;
+    double tail;
+    if (gxy <= room * turns) {
+      const double t = ts * (double)((gxy + room - 1) / room);
+      tail = t > last ? t : last;
+    } else {
+      tail = last + ts * (double)((gxy - room * turns + slots - 1) / slots);
+    }
+    const double alone = per_sm > 1 && full + gxy <= nsm ? 0.73 : 1.0;
+    const double cost = alone * ((double)waves * tf + tail);
     if (cost < best_cost - 1e-9) {
       best_cost = cost;
       best = kz;
