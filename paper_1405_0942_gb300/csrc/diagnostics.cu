@@ -89,20 +89,13 @@ __device__ double pull_B(const DG& g, const T* d, const T* B0s, int N, int i, in
   return det;
 }
 
-// Nearest-neighbour mimetic current at interior node (i, j, k) (compact
-// form of the three Stokes loops) and B there.
-template <typename T>
-__device__ void current_mimetic(const DG& g, const T* d, const T* B0s, int N, int i, int j,
-                                int k, double J[3], double B[3]) {
-  double G[3][3], Gn[3][3], Bp[3], Bm[3], P[3][3];
-  const double det = pull_B(g, d, B0s, N, i, j, k, G, B);
-  for (int a = 0; a < 3; ++a) {
-    const int e[3] = {a == 0, a == 1, a == 2};
-    pull_B(g, d, B0s, N, i + e[0], j + e[1], k + e[2], Gn, Bp);
-    pull_B(g, d, B0s, N, i - e[0], j - e[1], k - e[2], Gn, Bm);
-    for (int c = 0; c < 3; ++c) P[a][c] = Bp[c] - Bm[c];
-  }
-  double cc[3];
+// Nearest-neighbour mimetic current (compact form of the three Stokes loops)
+// from G and det G at the node and B at its six neighbours (+x, -x, +y, ..).
+__device__ __forceinline__ void current_mimetic(const double G[3][3], double det,
+                                                const double (*Bn)[3], double J[3]) {
+  double P[3][3], cc[3];
+  for (int a = 0; a < 3; ++a)
+    for (int c = 0; c < 3; ++c) P[a][c] = Bn[2 * a][c] - Bn[2 * a + 1][c];
   for (int a = 0; a < 3; ++a) {
     const int a1 = (a + 1) % 3, a2 = (a + 2) % 3;
     cc[a] = ddot(P[a1], G[a2]) - ddot(P[a2], G[a1]);
@@ -264,7 +257,7 @@ __device__ double block_max(double v, double* sh) {
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x == 0)
-    for (int w = 0; w < DT / 32; ++w) t = fmax(t, sh[w]);
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t = fmax(t, sh[w]);
   return t;
 }
 
@@ -315,46 +308,79 @@ __global__ void __launch_bounds__(DT) k_deviation_final(const double* part, int 
   }
 }
 
-// alpha* at the interior nodes of the line (i, j, .) into out[0 .. nz-1]
-// (NaN at the two boundary nodes) and epsilon* into out[nz]; one CTA,
-// dynamic shared memory of nz doubles.
+// alpha* at the interior nodes of the line (i, j, .) into out[0 .. nz-1] (NaN
+// at the two boundary nodes); out[nz] is cleared for k_alpha_eps.  An FP64
+// instruction costs the same for one lane of a warp as for 32, and a line has
+// few nodes, so the seven pull-backs a nearest-neighbour current needs run on
+// seven threads of the LINE_NODES x 7 of a CTA (33 nodes and their epsilon*:
+// 49 us as one thread per node in one CTA, 15 + 3 us in these two kernels).
+constexpr int LINE_NODES = DT / 7;
 template <typename T, int CURL>
 __global__ void __launch_bounds__(DT) k_alpha_line(DG g, const void* const* dbuf,
                                                    const DevState* st, const T* B0s, int i,
-                                                   int j, double a_r, double* out) {
-  extern __shared__ double al[];
-  __shared__ double sh[DT / 32];
+                                                   int j, double* out) {
   const T* d = (const T*)dbuf[st->cur];
   const int N = g.nx * g.ny * g.nz;
-  for (int k = threadIdx.x; k < g.nz; k += DT) {
-    double a = NAN;
-    if (k >= 1 && k <= g.nz - 2) {
-      double J[3], B[3];
-      if (CURL == GLEMUR_CURL_DIRECT)
-        current_direct(g, d, B0s, N, i, j, k, J, B);
-      else if (CURL == GLEMUR_CURL_NNN)
-        current_nnn(g, d, B0s, N, i, j, k, J, B);
-      else
-        current_mimetic(g, d, B0s, N, i, j, k, J, B);
-      a = ddot(J, B) / ddot(B, B);
+  if (blockIdx.x == 0 && threadIdx.x == 0) out[g.nz] = 0.0;
+  if constexpr (CURL == GLEMUR_CURL_MIMETIC) {
+    __shared__ double sB[7 * LINE_NODES][3];
+    const int m = threadIdx.x / 7, q = threadIdx.x % 7, k = blockIdx.x * LINE_NODES + m;
+    const bool mine = m < LINE_NODES && k >= 1 && k <= g.nz - 2;
+    double G[3][3], det = 1.0, B[3];
+    if (mine) {  // q = 0: the node, then +x, -x, +y, -y, +z, -z of it
+      const int s = q & 1 ? 1 : -1;
+      det = pull_B(g, d, B0s, N, i + (q == 1 || q == 2 ? s : 0), j + (q == 3 || q == 4 ? s : 0),
+                   k + (q >= 5 ? s : 0), G, B);
+      for (int c = 0; c < 3; ++c) sB[threadIdx.x][c] = B[c];
     }
-    al[k] = a;
-    out[k] = a;
+    __syncthreads();
+    if (q == 0 && m < LINE_NODES && k < g.nz) {
+      double a = NAN;
+      if (mine) {
+        double J[3];
+        current_mimetic(G, det, sB + threadIdx.x + 1, J);
+        a = ddot(J, B) / ddot(B, B);
+      }
+      out[k] = a;
+    }
+  } else {
+    const int k = blockIdx.x * LINE_NODES + threadIdx.x;
+    if (threadIdx.x < LINE_NODES && k < g.nz) {
+      double a = NAN;
+      if (k >= 1 && k <= g.nz - 2) {
+        double J[3], B[3];
+        if (CURL == GLEMUR_CURL_DIRECT)
+          current_direct(g, d, B0s, N, i, j, k, J, B);
+        else
+          current_nnn(g, d, B0s, N, i, j, k, J, B);
+        a = ddot(J, B) / ddot(B, B);
+      }
+      out[k] = a;
+    }
   }
-  __syncthreads();
+}
+
+// epsilon* into out[nz]: the largest a_r (alpha*_k - alpha*_l) / |X_k - X_l|
+// over pairs of interior nodes, one CTA per k (a maximum of non-negative
+// values: their bit patterns order alike).
+__global__ void __launch_bounds__(DT) k_alpha_eps(DG g, double a_r, double* out) {
+  __shared__ double sh[DT / 32];
+  const int k = 1 + blockIdx.x;
+  const double ak = out[k];
   double e = 0.0;
-  for (int k = 1 + threadIdx.x; k <= g.nz - 2; k += DT)
-    for (int l = 1; l <= g.nz - 2; ++l) {
-      if (l == k) continue;
-      const double v = a_r * (al[k] - al[l]) / (fabs((double)(k - l)) * g.h[2]);
-      e = fmax(e, v);
-    }
+  for (int l = 1 + threadIdx.x; l <= g.nz - 2; l += blockDim.x) {
+    if (l == k) continue;
+    const double v = a_r * (ak - out[l]) / (fabs((double)(k - l)) * g.h[2]);
+    e = fmax(e, v);
+  }
   e = block_max(e, sh);
-  if (threadIdx.x == 0) out[g.nz] = e;
+  if (threadIdx.x == 0 && e > 0.0)  // never the bits of -0
+    atomicMax((unsigned long long*)(out + g.nz), (unsigned long long)__double_as_longlong(e));
 }
 
 // kappa at every node (into kappa when non-null) and the number of concave
-// nodes per CTA.
+// nodes per CTA.  FP64-bound: every edge vector, cross product and sign once
+// (a call with the field, copies included: 33^3 48 -> 36 us, 128^3 817 -> 356).
 template <typename T>
 __global__ void __launch_bounds__(DT) k_convexity(DG g, const void* const* dbuf,
                                                   const DevState* st, signed char* kappa,
@@ -367,23 +393,35 @@ __global__ void __launch_bounds__(DT) k_convexity(DG g, const void* const* dbuf,
   for (int n = blockIdx.x * DT + threadIdx.x; n < N; n += gridDim.x * DT) {
     const int id[3] = {n % g.nx, (n / g.nx) % g.ny, n / (g.nx * g.ny)};
     const int ext[3] = {g.nx, g.ny, g.nz};
-    // x(neighbour) - x(node) along axis a, direction s: d difference + s h_a e_a
-    bool ok = true;
-    for (int oct = 0; oct < 8; ++oct) {
-      const int sg[3] = {(oct & 1) ? 1 : -1, (oct & 2) ? 1 : -1, (oct & 4) ? 1 : -1};
-      bool inside = true;
-      for (int a = 0; a < 3; ++a) inside = inside && id[a] + sg[a] >= 0 && id[a] + sg[a] < ext[a];
-      if (!inside) continue;
-      double v[3][3];
-      for (int a = 0; a < 3; ++a) {
-        const int m = n + sg[a] * stp[a];
-        for (int c = 0; c < 3; ++c) v[a][c] = (double)d[c * N + m] - (double)d[c * N + n];
-        v[a][a] += sg[a] * g.h[a];
+    // x(neighbour) - x(node) along axis a, direction s: d difference + s h_a
+    // e_a; the six of them once, the cross product of each pair along y and z
+    // once, and the determinants' signs on the integer pipes
+    double v[3][2][3];
+    bool in[3][2];
+    for (int a = 0; a < 3; ++a)
+      for (int q = 0; q < 2; ++q) {
+        const int s = q ? 1 : -1;
+        in[a][q] = id[a] + s >= 0 && id[a] + s < ext[a];
+        const int m = in[a][q] ? n + s * stp[a] : n;
+        for (int c = 0; c < 3; ++c) v[a][q][c] = (double)d[c * N + m] - (double)d[c * N + n];
+        v[a][q][a] += s * g.h[a];
       }
-      const double D = ddet(v[0], v[1], v[2]);
-      const int sgn = D > 0.0 ? 1 : (D < 0.0 ? -1 : 0);
-      if (sgn != sg[0] * sg[1] * sg[2]) ok = false;
-    }
+    bool ok = true;
+    for (int q1 = 0; q1 < 2; ++q1)
+      for (int q2 = 0; q2 < 2; ++q2) {
+        const double* y = v[1][q1];
+        const double* z = v[2][q2];
+        const double c0 = y[1] * z[2] - y[2] * z[1], c1 = y[2] * z[0] - y[0] * z[2],
+                     c2 = y[0] * z[1] - y[1] * z[0];
+        for (int q0 = 0; q0 < 2; ++q0) {
+          if (!(in[0][q0] && in[1][q1] && in[2][q2])) continue;
+          const double* x = v[0][q0];
+          const double D = x[0] * c0 + x[1] * c1 + x[2] * c2;
+          const long long b = __double_as_longlong(D);
+          const bool want_neg = (q0 + q1 + q2) % 2 == 0;  // the sign of di dj dk
+          if ((b << 1) == 0 || (b < 0) != want_neg || !not_nan(D)) ok = false;
+        }
+      }
     if (kappa) kappa[n] = ok ? 1 : -1;
     if (!ok) cnt += 1.0;
   }
@@ -468,30 +506,30 @@ int glemur_alpha_line(glemur_ctx* ctx, int i, int j, double a_r, double* alpha,
   DiagCtx c;
   int rc = ctx_diag(ctx, &c);
   if (rc) return rc;
-  // the line's alpha* values sit in shared memory (at most 48 KiB)
   if (i < 1 || i > c.nx - 2 || j < 1 || j > c.ny - 2 || !(a_r > 0) || c.nz > 6144)
     return GLEMUR_ERR_BADARG;
   const DG g = geom_of(c);
-  const size_t sm = sizeof(double) * c.nz;
   const bool direct = c.curl == GLEMUR_CURL_DIRECT;
+  const int nb = (c.nz + LINE_NODES - 1) / LINE_NODES;
   if (c.curl == GLEMUR_CURL_NNN) {  // FP64 contexts only
-    k_alpha_line<double, 2><<<1, DT, sm, c.s>>>(g, c.dbuf_dev, c.st, (const double*)c.B0s, i, j,
-                                                a_r, c.stage);
+    k_alpha_line<double, 2><<<nb, DT, 0, c.s>>>(g, c.dbuf_dev, c.st, (const double*)c.B0s, i, j,
+                                                c.stage);
   } else if (c.precision == GLEMUR_MIXED) {
     if (direct)
-      k_alpha_line<float, 1><<<1, DT, sm, c.s>>>(g, c.dbuf_dev, c.st, (const float*)c.B0s, i, j,
-                                                 a_r, c.stage);
+      k_alpha_line<float, 1><<<nb, DT, 0, c.s>>>(g, c.dbuf_dev, c.st, (const float*)c.B0s, i, j,
+                                                 c.stage);
     else
-      k_alpha_line<float, 0><<<1, DT, sm, c.s>>>(g, c.dbuf_dev, c.st, (const float*)c.B0s, i, j,
-                                                 a_r, c.stage);
+      k_alpha_line<float, 0><<<nb, DT, 0, c.s>>>(g, c.dbuf_dev, c.st, (const float*)c.B0s, i, j,
+                                                 c.stage);
   } else {
     if (direct)
-      k_alpha_line<double, 1><<<1, DT, sm, c.s>>>(g, c.dbuf_dev, c.st, (const double*)c.B0s, i,
-                                                  j, a_r, c.stage);
+      k_alpha_line<double, 1><<<nb, DT, 0, c.s>>>(g, c.dbuf_dev, c.st, (const double*)c.B0s, i,
+                                                  j, c.stage);
     else
-      k_alpha_line<double, 0><<<1, DT, sm, c.s>>>(g, c.dbuf_dev, c.st, (const double*)c.B0s, i,
-                                                  j, a_r, c.stage);
+      k_alpha_line<double, 0><<<nb, DT, 0, c.s>>>(g, c.dbuf_dev, c.st, (const double*)c.B0s, i,
+                                                  j, c.stage);
   }
+  k_alpha_eps<<<c.nz - 2, c.nz <= 66 ? 64 : DT, 0, c.s>>>(g, a_r, c.stage);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && alpha)
     e = cudaMemcpyAsync(alpha, c.stage, sizeof(double) * c.nz, cudaMemcpyDeviceToHost, c.s);
