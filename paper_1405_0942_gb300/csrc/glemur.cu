@@ -126,55 +126,149 @@ __device__ __forceinline__ double label(const GridGeom& g, int a, int i) {
   return g.lo[a] + (double)i * g.h[a];
 }
 
+// The FP64 pipe takes a warp's double <-> float conversion, like any FP64
+// instruction, in 64 cycles per SM quarter; as integer operations they are
+// about ten of two cycles.  Rounding is to nearest even, as a cast's; zeros,
+// and what is not a normal float on both sides, go through the cast.
+__device__ __forceinline__ void narrow(double v, double& o) { o = v; }
+__device__ __forceinline__ void narrow(double v, float& o) {
+  const long long b = __double_as_longlong(v);
+  const unsigned hi = (unsigned)(b >> 32), e = (hi >> 20) & 0x7ff;
+  if (e - 897u < 254u) {
+    unsigned long long m = ((unsigned long long)b & 0x7fffffffffffffffull) - (896ull << 52);
+    m += 0x0fffffff + ((m >> 29) & 1);
+    o = __uint_as_float((unsigned)(m >> 29) | (hi & 0x80000000u));
+  } else if ((b << 1) == 0) {
+    o = __uint_as_float(hi);
+  } else {
+    o = (float)v;
+  }
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+  const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+  const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
+  if (m - 0x00800000u < 0x7f000000u)
+    return __longlong_as_double((long long)(sign | (((unsigned long long)m << 29) + (896ull << 52))));
+  if (m == 0) return __longlong_as_double((long long)sign);
+  return (double)v;
+}
+
+// Conversions of whole fields: a thread takes a node of the (x, y) plane and
+// up to CONV_PLANES planes of it, so that the node labels (a conversion and
+// an FMA on the FP64 pipe each) cost a few of its instructions per column,
+// with CONV_BATCH planes' loads in flight.  Small grids take fewer planes per
+// CTA, so that every SM has one (16^3 with 8 planes, two CTAs: a call of
+// set_x takes 13.8 us, with one plane 11.8).
+constexpr int CONV_T = 256, CONV_PLANES = 8, CONV_BATCH = 4;
+struct Column {
+  int p, k0, k1;  // node of the plane, planes [k0, k1)
+};
+__device__ __forceinline__ Column conv_column(const GridGeom& g, int planes) {
+  const int cb = (g.nx * g.ny + CONV_T - 1) / CONV_T;
+  const int k0 = (int)(blockIdx.x / cb) * planes;
+  return {(int)(blockIdx.x % cb) * CONV_T + (int)threadIdx.x, k0, min(k0 + planes, g.nz)};
+}
+struct ConvGrid {
+  int planes, blocks;
+};
+ConvGrid conv_grid(int nx, int ny, int nz, int nsm) {
+  const int cb = (nx * ny + CONV_T - 1) / CONV_T;
+  int planes = CONV_PLANES;
+  while (planes > 1 && (long long)cb * ((nz + planes - 1) / planes) < nsm) planes /= 2;
+  return {planes, cb * ((nz + planes - 1) / planes)};
+}
+
+// d = x - X into the current displacements, and into the boundary nodes of
+// the other displacement buffer and of both stage inputs: the stages write
+// every interior node of these before they read it, and no boundary node.
+// Of 72 B per node of a mixed field that leaves the 36 of x and d, and of 12
+// FP64 instructions 3 (a call at 384^3: 1.28 -> 0.42 ms, HBM's share 0.30;
+// 256^3 in FP64 324 -> 160 us).  Grids hold fewer than 2^31 / 3 nodes, so
+// 32-bit indices suffice.
 template <typename T>
-// d = x - X into both displacement buffers and both stage-input buffers
-// (whose boundary entries must hold the fixed boundary positions).  Grids
-// hold fewer than 2^31 / 3 nodes, so 32-bit indices suffice.
-__global__ void k_set_x(GridGeom g, const double* __restrict__ x, T* d0, T* d1, T* y0, T* y1) {
-  const int N = g.nx * g.ny * g.nz;
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
-    const int i = n % g.nx, r = n / g.nx, j = r % g.ny, k = r / g.ny;
-    // periodic in z: a ghost plane takes its partner's displacement (the
-    // ghost's position is the partner's shifted by the period)
-    const int ks = g.periodic && k == 0 ? g.nz - 2 : (g.periodic && k == g.nz - 1 ? 1 : k);
-    const int ns = (ks * g.ny + j) * g.nx + i;
-    const double X[3] = {label(g, 0, i), label(g, 1, j), label(g, 2, ks)};
-    for (int c = 0; c < 3; ++c) {
-      const T v = (T)(x[c * N + ns] - X[c]);
-      d0[c * N + n] = v;
-      d1[c * N + n] = v;
-      y0[c * N + n] = v;
-      y1[c * N + n] = v;
+__global__ void __launch_bounds__(CONV_T) k_set_x(GridGeom g, int planes,
+                                                  const double* __restrict__ x, T* d0, T* d1, T* y0, T* y1) {
+  __shared__ double Z[CONV_PLANES];
+  const Column w = conv_column(g, planes);
+  const int nxy = g.nx * g.ny, N = nxy * g.nz;
+  // periodic in z: a ghost plane takes its partner's displacement (the
+  // ghost's position is the partner's shifted by the period)
+  auto source = [&](int k) {
+    return g.periodic && k == 0 ? g.nz - 2 : (g.periodic && k == g.nz - 1 ? 1 : k);
+  };
+  if (threadIdx.x < CONV_PLANES) Z[threadIdx.x] = label(g, 2, source(w.k0 + threadIdx.x));
+  __syncthreads();
+  if (w.p >= nxy) return;
+  const int i = w.p % g.nx, j = w.p / g.nx;
+  const double X = label(g, 0, i), Y = label(g, 1, j);
+  const bool side = i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1;
+  for (int kb = w.k0; kb < w.k1; kb += CONV_BATCH) {
+    double v[CONV_BATCH][3];
+#pragma unroll
+    for (int q = 0; q < CONV_BATCH; ++q)
+      if (kb + q < w.k1) {
+        const int n = source(kb + q) * nxy + w.p;
+        for (int c = 0; c < 3; ++c) v[q][c] = x[c * N + n];
+      }
+#pragma unroll
+    for (int q = 0; q < CONV_BATCH; ++q) {
+      const int k = kb + q;
+      if (k >= w.k1) break;
+      const int n = k * nxy + w.p;
+      const double L[3] = {X, Y, Z[k - w.k0]};
+      T d[3];
+      for (int c = 0; c < 3; ++c) {
+        narrow(v[q][c] - L[c], d[c]);
+        d0[c * N + n] = d[c];
+      }
+      if (side || k == 0 || k == g.nz - 1)
+        for (int c = 0; c < 3; ++c) d1[c * N + n] = y0[c * N + n] = y1[c * N + n] = d[c];
     }
   }
 }
 
+// x = X + d (384^3 mixed: 1.25 -> 0.45 ms; 256^3 in FP64 287 -> 148 us)
 template <typename T>
-__global__ void k_get_x(GridGeom g, const T* const* dbuf, const DevState* st,
-                        double* __restrict__ x) {
-  const int N = g.nx * g.ny * g.nz;
-  const T* d = dbuf[st->cur];
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
-    const int i = n % g.nx, r = n / g.nx, j = r % g.ny, k = r / g.ny;
-    const double X[3] = {label(g, 0, i), label(g, 1, j), label(g, 2, k)};
-    for (int c = 0; c < 3; ++c) x[c * N + n] = X[c] + (double)d[c * N + n];
+__global__ void __launch_bounds__(CONV_T) k_get_x(GridGeom g, int planes,
+                                                  const T* const* dbuf, const DevState* st,
+                                                  double* __restrict__ x) {
+  __shared__ double Z[CONV_PLANES];
+  const Column w = conv_column(g, planes);
+  const int nxy = g.nx * g.ny, N = nxy * g.nz;
+  const T* __restrict__ d = dbuf[st->cur];
+  if (threadIdx.x < CONV_PLANES) Z[threadIdx.x] = label(g, 2, w.k0 + threadIdx.x);
+  __syncthreads();
+  if (w.p >= nxy) return;
+  const double X = label(g, 0, w.p % g.nx), Y = label(g, 1, w.p / g.nx);
+#pragma unroll CONV_PLANES
+  for (int q = 0; q < CONV_PLANES; ++q) {
+    const int k = w.k0 + q;
+    if (k >= w.k1) break;
+    const int n = k * nxy + w.p;
+    const double L[3] = {X, Y, Z[q]};
+    for (int c = 0; c < 3; ++c) x[c * N + n] = L[c] + widen(d[c * N + n]);
   }
 }
 
+// B0s_a = B0_a * 4 h_{a+1} h_{a+2} (the factors s; 384^3 mixed: 0.63 -> 0.38 ms)
 template <typename T>
-__global__ void k_set_B0(GridGeom g, const double* __restrict__ B0, T* B0s) {
-  const int N = g.nx * g.ny * g.nz;
-  // B0s_a = B0_a * 4 h_{a+1} h_{a+2}
-  const double s[3] = {4.0 * g.h[1] * g.h[2], 4.0 * g.h[2] * g.h[0], 4.0 * g.h[0] * g.h[1]};
+__global__ void k_set_B0(int N, const double* __restrict__ B0, T* __restrict__ B0s, double s0,
+                         double s1, double s2) {
+  const double s[3] = {s0, s1, s2};
   for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x)
-    for (int c = 0; c < 3; ++c) B0s[c * N + n] = (T)(B0[c * N + n] * s[c]);
+    for (int c = 0; c < 3; ++c) {
+      T v;
+      narrow(B0[c * N + n] * s[c], v);
+      B0s[c * N + n] = v;
+    }
 }
 
 template <typename T>
 __global__ void k_to_f64(long long M, const T* __restrict__ src, double* __restrict__ dst) {
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < M;
        n += (long long)gridDim.x * blockDim.x)
-    dst[n] = (double)src[n];
+    dst[n] = widen(src[n]);
 }
 
 }  // namespace glemur
@@ -1045,14 +1139,15 @@ int glemur_set_x(glemur_ctx* c, const double* x, int mem) {
   const double* src = nullptr;
   int rc = stage_in(c, x, mem, &src);
   if (rc) return rc;
-  const int nb = elementwise_blocks(c->N);
+  const ConvGrid cg = conv_grid(c->nx, c->ny, c->nz, c->nsm);
   if (c->o.precision == GLEMUR_MIXED)
-    k_set_x<float><<<nb, 256, 0, c->s>>>(geom(c), src, (float*)c->dbuf[0], (float*)c->dbuf[1],
-                                         (float*)c->ys[0], (float*)c->ys[1]);
+    k_set_x<float><<<cg.blocks, CONV_T, 0, c->s>>>(
+        geom(c), cg.planes, src, (float*)c->dbuf[0], (float*)c->dbuf[1], (float*)c->ys[0],
+        (float*)c->ys[1]);
   else
-    k_set_x<double><<<nb, 256, 0, c->s>>>(geom(c), src, (double*)c->dbuf[0],
-                                          (double*)c->dbuf[1], (double*)c->ys[0],
-                                          (double*)c->ys[1]);
+    k_set_x<double><<<cg.blocks, CONV_T, 0, c->s>>>(
+        geom(c), cg.planes, src, (double*)c->dbuf[0], (double*)c->dbuf[1], (double*)c->ys[0],
+        (double*)c->ys[1]);
   rc = cuda_rc(cudaGetLastError());
   if (rc) return rc;
   return reset_state(c);  // k_set_x also seeded the stage inputs
@@ -1087,23 +1182,26 @@ int glemur_set_B0(glemur_ctx* c, const double* B0, int mem) {
   const double* src = nullptr;
   int rc = stage_in(c, B0, mem, &src);
   if (rc) return rc;
-  const int nb = elementwise_blocks(c->N);
+  const int nb = elementwise_blocks(c->N), N = (int)c->N;
+  const double* h = c->h;
+  const double s[3] = {4.0 * h[1] * h[2], 4.0 * h[2] * h[0], 4.0 * h[0] * h[1]};
   if (c->o.precision == GLEMUR_MIXED)
-    k_set_B0<float><<<nb, 256, 0, c->s>>>(geom(c), src, (float*)c->B0s);
+    k_set_B0<float><<<nb, 256, 0, c->s>>>(N, src, (float*)c->B0s, s[0], s[1], s[2]);
   else
-    k_set_B0<double><<<nb, 256, 0, c->s>>>(geom(c), src, (double*)c->B0s);
+    k_set_B0<double><<<nb, 256, 0, c->s>>>(N, src, (double*)c->B0s, s[0], s[1], s[2]);
   return cuda_rc(cudaGetLastError());
 }
 
 int glemur_get_x(glemur_ctx* c, double* x, int mem) {
   if (!c || !x || (mem != GLEMUR_MEM_DEVICE && mem != GLEMUR_MEM_HOST)) return GLEMUR_ERR_BADARG;
   double* dst = out_target(c, x, mem);
-  const int nb = elementwise_blocks(c->N);
+  const ConvGrid cg = conv_grid(c->nx, c->ny, c->nz, c->nsm);
   if (c->o.precision == GLEMUR_MIXED)
-    k_get_x<float><<<nb, 256, 0, c->s>>>(geom(c), (const float* const*)c->dbuf_dev, c->st, dst);
+    k_get_x<float><<<cg.blocks, CONV_T, 0, c->s>>>(
+        geom(c), cg.planes, (const float* const*)c->dbuf_dev, c->st, dst);
   else
-    k_get_x<double><<<nb, 256, 0, c->s>>>(geom(c), (const double* const*)c->dbuf_dev, c->st,
-                                          dst);
+    k_get_x<double><<<cg.blocks, CONV_T, 0, c->s>>>(
+        geom(c), cg.planes, (const double* const*)c->dbuf_dev, c->st, dst);
   int rc = cuda_rc(cudaGetLastError());
   if (rc) return rc;
   return stage_out(c, x, dst, mem);
