@@ -360,10 +360,11 @@ size_t glemur_adjoint_segment_bytes(glemur_ctx* ctx, int n_steps, int every);
  * controlled run recorded, glemur_get_dt_schedule), into *value, and its
  * gradients: with respect to x0 into lam_x0 and with respect to B0 into
  * mu_B0 (device float64 fields, overwritten).  Forward: glemur_set_x(x0),
- * then the steps, keeping the raw state every `every` steps in seg_ws;
- * backward: each segment recomputed forwards from its checkpoint with its
- * states kept, the loss gradient seeded at the final state, and the steps'
- * glemur_vjp_step in reverse -- checkpointing with recompute, memory
+ * then the steps, keeping the raw state every `every` steps and those within
+ * the last segment in seg_ws; backward: the loss gradient seeded at the final
+ * state, each earlier segment recomputed forwards from its checkpoint up to
+ * its last step with its states kept, and the steps' glemur_vjp_step in
+ * reverse -- checkpointing with recompute, memory
  * O(n_steps/every + every) states.  x0 must not alias the workspaces (it
  * may be lam_x0 or mu_B0: it is read before they are written);
  * seg_ws (256-byte aligned, glemur_adjoint_segment_bytes) and adj_ws (as

@@ -998,12 +998,14 @@ int glemur_adjoint_segment(glemur_ctx* c, const double* x0, const double* dts, i
   const size_t F3 = sizeof(double) * 3 * (size_t)nx * ny * nz;
   const long long nseg = n > 0 ? ((long long)n + every - 1) / every : 1;
   const int per = n < every ? n : every;
+  const int last = (int)((nseg - 1) * every);  // first step of the last segment
   unsigned char* base = (unsigned char*)seg_ws;
-  unsigned char* states = base + (size_t)nseg * S;  // the states after each step of a segment
+  unsigned char* states = base + (size_t)nseg * S;  // the states between a segment's steps
   double* scratch = (double*)(states + (size_t)per * S);
   auto ckpt = [&](long long q) { return (void*)(base + (size_t)q * S); };
-  // forward: checkpoints at steps 0, every, 2 every, ... (< n); x0 is read
-  // before the outputs are cleared, so it may share a buffer with them
+  // forward: checkpoints at steps 0, every, 2 every, ... (< n), and the
+  // states between the last segment's steps, which are reversed next; x0 is
+  // read before the outputs are cleared, so it may share a buffer with them
   glemur_stats st;
   if ((rc = glemur_set_x(c, x0, GLEMUR_MEM_DEVICE))) return rc;
   if ((rc = glemur_get_state(c, ckpt(0)))) return rc;
@@ -1013,8 +1015,9 @@ int glemur_adjoint_segment(glemur_ctx* c, const double* x0, const double* dts, i
   if (e != cudaSuccess) return GLEMUR_ERR_CUDA;
   for (int i = 0; i < n; ++i) {
     if ((rc = glemur_step_fixed(c, dts[i], &st))) return rc;
-    if ((i + 1) % every == 0 && i + 1 < n && (rc = glemur_get_state(c, ckpt((i + 1) / every))))
-      return rc;
+    if (i + 1 == n) break;  // the final state seeds the reverse pass from the context
+    if ((i + 1) % every == 0 && (rc = glemur_get_state(c, ckpt((i + 1) / every)))) return rc;
+    if (i >= last && (rc = glemur_get_state(c, states + (size_t)(i - last) * S))) return rc;
   }
   if (n == 0) {
     if ((rc = glemur_set_state(c, ckpt(0)))) return rc;
@@ -1026,10 +1029,15 @@ int glemur_adjoint_segment(glemur_ctx* c, const double* x0, const double* dts, i
   bool seeded = false;
   for (long long q = nseg - 1; q >= 0; --q) {
     const int start = (int)(q * every), end = start + every < n ? start + every : n;
-    if ((rc = glemur_set_state(c, ckpt(q)))) return rc;
-    for (int i = start; i < end; ++i) {
-      if ((rc = glemur_step_fixed(c, dts[i], &st))) return rc;
-      if ((rc = glemur_get_state(c, states + (size_t)(i - start) * S))) return rc;
+    // the states between its steps: the last segment's are kept already, and
+    // no segment's last step is needed (64^3, four steps, a checkpoint every
+    // two: one step repeated instead of four, 7.30 -> 6.28 ms)
+    if (start != last && end - start > 1) {
+      if ((rc = glemur_set_state(c, ckpt(q)))) return rc;
+      for (int i = start; i + 1 < end; ++i) {
+        if ((rc = glemur_step_fixed(c, dts[i], &st))) return rc;
+        if ((rc = glemur_get_state(c, states + (size_t)(i - start) * S))) return rc;
+      }
     }
     if (!seeded) {  // the context is at the final state
       if ((rc = glemur_loss_grad(c, loss, value, lam_next, mu_B0, adj_ws, adj_bytes))) return rc;
