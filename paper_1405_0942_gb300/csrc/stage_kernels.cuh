@@ -1,4 +1,8 @@
-// Fused Cash-Karp stage kernels for the Lagrangian magneto-frictional step.
+// Fused Cash-Karp stage kernels for the Lagrangian magneto-frictional step:
+// the direct current's in mixed precision, and the mimetic current's in FP64
+// where GLEMUR_F64_FUSED asks for it (the FP64 passes of kern_f64_split.cu and
+// kern_f64_direct.cu and the mixed mimetic march of stage_march.cuh are faster
+// for the rest; they share the arithmetic below).
 //
 // One launch evaluates one Runge-Kutta stage k_s = u(x_s) at every interior
 // node (section "Time Stepping"; eq. "x integration" with u = J x B of eq.

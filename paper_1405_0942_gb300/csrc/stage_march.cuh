@@ -22,8 +22,9 @@
 // global accesses, and share every index, branch and barrier: 344 issue
 // slots per node in stage 4 where one node per thread on 32-wide tiles took
 // 542 with the same carried registers, and 564 re-reading G and B from
-// shared memory.  An attempt: 384^3 7.16 -> 4.87 ms, 128^3 351 -> 255 us,
-// 48^3 70 -> 59 us, 101 x 90 x 75 (plain copies) 197 -> 174 us.  Measured and
+// shared memory.  An attempt: 384^3 7.16 -> 4.87 ms, 128^3 351 -> 243 us,
+// 48^3 70 -> 59 us, 101 x 90 x 75 (plain copies) 197 -> 159 us (the last 12
+// and 15 us by choose_kz_march's planes per CTA).  Measured and
 // left: one column per thread (384^3 6.2 ms at 24 warps per SM, 6.5 ms at
 // 16), 16 or 4 warps per CTA (5.7, 5.6 ms).  128 registers, 2 CTAs per SM.
 //
