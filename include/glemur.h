@@ -161,7 +161,7 @@ size_t glemur_workspace_bytes(int nx, int ny, int nz, int precision);
  *                         whole attempts (twelve passes and the control) in
  *                         one persistent cooperative launch with per-plane
  *                         waits instead of one launch per pass (same
- *                         results bit for bit; measured 14 % slower at 64^3)
+ *                         results bit for bit; measured 12 % slower at 64^3)
  *   GLEMUR_TEST_PERSIST_TIMEOUT=1  test hook: in the persistent launch one
  *                         CTA never reports a finished pass, so the bounded
  *                         waits of its neighbours give up after 2 s and

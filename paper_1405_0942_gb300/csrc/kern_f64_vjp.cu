@@ -19,10 +19,10 @@
 //              nodes those of node p are the central ones at p -+ 1, weight
 //              +-1, or on a face the one-sided one, weight +-4, and the
 //              one-sided one two nodes away, weight -+1.
-// 217 FP64 instructions per node and stage, where forming G again in both of
-// the first two passes, B0s's product in the second and every k's adjoint in
-// the third took 286; pull-back 64 -> 43 us at 64^3; the gradient over four
-// steps there 8.27 -> 7.34 ms.
+// 242 FP64-pipe instructions per interior node and stage (120 + 82 + 39),
+// without forming G again in the first two passes, B0s's product in the
+// second and every k's adjoint in the third; pull-back 64 -> 43 us at 64^3;
+// the gradient over four steps there 8.27 -> 7.34 ms.
 #include "split64.cuh"
 #include "vjp64.cuh"
 
