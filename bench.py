@@ -60,14 +60,14 @@ MIN_TIMED_S = 1.0              # repeat the block of timed attempts until this
 # captured from (kernel_source_hash()); a workload without an entry, or one
 # whose kernels have changed since, reports null
 NCU_TRAFFIC = {
-    ("braid64", "fp64", "mimetic"): (57728554, "f0b96345d86b"),
-    ("braid64", "fp64", "direct"): (31320234, "f0b96345d86b"),
-    ("braid64", "fp64", "nnn"): (43997056, "f0b96345d86b"),
-    ("periodic64", "fp64", "mimetic"): (57531904, "f0b96345d86b"),
-    ("braid64", "mixed", "mimetic"): (15672277, "f0b96345d86b"),
-    ("braid64", "mixed", "direct"): (15829333, "f0b96345d86b"),
-    ("braid128", "mixed", "mimetic"): (152607573, "f0b96345d86b"),
-    ("prod384", "mixed", "mimetic"): (4721120981, "f0b96345d86b"),
+    ("braid64", "fp64", "mimetic"): (57728170, "24b69e0a665f"),
+    ("braid64", "fp64", "direct"): (31325952, "24b69e0a665f"),
+    ("braid64", "fp64", "nnn"): (43994837, "24b69e0a665f"),
+    ("periodic64", "fp64", "mimetic"): (57529386, "24b69e0a665f"),
+    ("braid64", "mixed", "mimetic"): (15672149, "24b69e0a665f"),
+    ("braid64", "mixed", "direct"): (15830229, "24b69e0a665f"),
+    ("braid128", "mixed", "mimetic"): (152600405, "24b69e0a665f"),
+    ("prod384", "mixed", "mimetic"): (4722780842, "24b69e0a665f"),
 }
 
 

@@ -168,7 +168,8 @@ __device__ void control_block(DevState* st, const double* part, int nb, int diag
     } else if (replay) {
       accept = true;
     } else if (lam > lambda0) {
-      double fac = safety * fifth_root(lambda0 * recip(lam));
+      // (a division: Lambda may be subnormal, which recip does not take)
+      double fac = safety * fifth_root(lambda0 / lam);
       if (fac < shrink_min) fac = shrink_min;
       dtn = dt * fac;
       if (consec + 1 > max_rejects || dtn < dt_min) status = ST_DT_UNDERFLOW;
@@ -176,7 +177,7 @@ __device__ void control_block(DevState* st, const double* part, int nb, int diag
       accept = true;
       double fac = 1.0;
       if (lam < 0.5 * lambda0) {
-        fac = lam > 0.0 ? safety * fifth_root(lambda0 * recip(lam)) : grow_max;
+        fac = lam > 0.0 ? safety * fifth_root(lambda0 / lam) : grow_max;
         if (fac > grow_max) fac = grow_max;
       }
       dtn = dt * fac;

@@ -260,9 +260,11 @@ __device__ __forceinline__ long long nidx(int i, int j, int k, int nx, int ny) {
 // Handbook of Floating-Point Arithmetic, ch. on Newton-Raphson division),
 // so two steps take the approximation to within an ulp or two of the
 // correctly rounded 1/v in 4 FMAs, where the IEEE division costs about 12
-// FP64-pipe instructions -- a quarter of the FP64 work of forming B.  NaN
-// propagates; 0 and subnormal v give NaN or inf, and every caller has
-// already flagged det <= 0 (or tested v > 0 and takes inf for a limit).
+// FP64-pipe instructions -- a quarter of the FP64 work of forming B.  For
+// |v| in [2^-1022, 2^1022]: 0, subnormal v, inf and NaN give NaN, larger
+// finite v 0.  Its callers pass det G (a value <= 0 is flagged), det M of the
+// next-nearest-neighbour current (NaN where the loops are degenerate: the
+// error norm reports it) and y^4 of fifth_root (within [1e-24, 1e24]).
 __device__ __forceinline__ double recip(double v) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
