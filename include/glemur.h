@@ -156,7 +156,8 @@ size_t glemur_workspace_bytes(int nx, int ny, int nz, int precision);
  *   GLEMUR_F64_FUSED=1    FP64: single-kernel mimetic stages (halo
  *                         recomputation) instead of the two-pass stages
  *   GLEMUR_KZ=k           z-planes per CTA of the stage kernels instead of
- *                         the cost model's choice
+ *                         the cost model's choice (more where k are too few
+ *                         for a launch: 65535 slabs at most)
  *   GLEMUR_PERSIST=1      FP64 two-pass stages, line-tied, loop currents:
  *                         whole attempts (twelve passes and the control) in
  *                         one persistent cooperative launch with per-plane

@@ -494,6 +494,17 @@ int elementwise_blocks(long long n) {
   return (int)(b < 4096 ? (b < 1 ? 1 : b) : 4096);
 }
 
+// Planes per CTA along z: at least as many as keep the slabs of nz planes
+// within a launch's z extent.
+int least_kz(int nz) { return (nz + 65534) / 65535; }
+
+// GLEMUR_KZ's planes per CTA, 0 without one.
+int kz_from_env(int nz) {
+  const char* env = getenv("GLEMUR_KZ");
+  const int kz = env ? atoi(env) : 0, least = least_kz(nz);
+  return kz < 1 ? 0 : (kz > nz ? nz : (kz < least ? least : kz));
+}
+
 // Planes per CTA along z of the fused FP64 and the mixed direct stage kernels.
 // Cost model: the time of the busiest SM, in units of one B plane (a CTA of
 // kz planes computes kz + 2 B planes).  FP64 stages are bound by the SM's
@@ -501,13 +512,12 @@ int elementwise_blocks(long long n) {
 // (kz + 2); the FP32 stages are latency-bound, so up to `per_sm` co-resident
 // CTAs overlap and the time is waves x (kz + 2).
 int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe) {
-  const char* env = getenv("GLEMUR_KZ");
-  if (env && atoi(env) > 0) return atoi(env) < nz ? atoi(env) : nz;
+  if (const int kz = kz_from_env(nz)) return kz;
   if (nsm < 1) nsm = 1;
   if (per_sm < 1) per_sm = 1;
   int best = nz;
   double best_cost = 1e300;
-  for (int kz = 1; kz <= nz; ++kz) {
+  for (int kz = least_kz(nz); kz <= nz; ++kz) {
     const long long ctas = (long long)gxy * ((nz + kz - 1) / kz);
     const long long slots = shared_pipe ? nsm : (long long)nsm * per_sm;
     const double waves = (double)((ctas + slots - 1) / slots);
@@ -531,16 +541,17 @@ int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe) {
 // CTA per SM at most an iteration takes 0.73 as long as with two (64^3, kz =
 // 4, 2: 76, 70 us).  Long marches lose to short ones on grids of many waves
 // (384^3: kz = 28, 36, 48 take 4.89, 4.85, 4.91 ms, 192 takes 9 % more than
-// 32), hence the limit of 40.
+// 32), hence the limit of 40 -- more where 40 planes each are more slabs than
+// a launch counts along z (3 x 3 x 2621403).
 int choose_kz_march(int nz, int gxy, int nsm, int per_sm) {
-  const char* env = getenv("GLEMUR_KZ");
-  if (env && atoi(env) > 0) return atoi(env) < nz ? atoi(env) : nz;
+  if (const int kz = kz_from_env(nz)) return kz;
   if (nsm < 1) nsm = 1;
   if (per_sm < 1) per_sm = 1;
   const long long slots = (long long)nsm * per_sm;
+  const int least = least_kz(nz), most = least > 40 ? least : 40;
   int best = nz;
   double best_cost = 1e300;
-  for (int kz = 1; kz <= nz && kz <= 40; ++kz) {
+  for (int kz = least; kz <= nz && kz <= most; ++kz) {
     const long long slabs = (nz + kz - 1) / kz;
     const long long full = gxy * (slabs - 1), waves = full / slots, left = full % slots;
     const double tf = kz + 2.5, ts = (double)(nz - (slabs - 1) * kz) + 1.5;
