@@ -329,8 +329,9 @@ struct MarchCentre {
 // Current, velocity and the stage's outputs at the thread's pair of plane m:
 // the B plane bm there, P2 the z difference of B, G and 1/det G of plane m,
 // yc its stage input, i the pair's first element.  A pair's node on an
-// x face is written too, with velocity 0: k is 0 there, so its stage input
-// and update are the fixed boundary position again.
+// x face is written too, with velocity 0: k is 0 there, so its stage input is
+// the fixed boundary position again, and its update that position's bits (d +
+// 0 would turn a negative zero).
 template <class Gm, int S, bool VEC>
 __device__ __forceinline__ void march_out(const StageArgs<float>& a, const MarchPair& own,
                                           bool second, const float* __restrict__ bm,
@@ -394,7 +395,14 @@ __device__ __forceinline__ void march_out(const StageArgs<float>& a, const March
       const f2 up = f2fma(co[3], u[c], f2fma(co[2], k4, f2fma(co[1], k3, f2mul(co[0], k1))));
       const f2 er = f2fma(
           co[8], u[c], f2fma(co[7], k5, f2fma(co[6], k4, f2fma(co[5], k3, f2mul(co[4], k1)))));
-      march_st<VEC>(dout, i + c * N, second, f2add(ce.d[c], up));
+      f2 dn = f2add(ce.d[c], up);
+      if (own.xface()) {
+        float d0, d1, n0, n1;
+        f2split(ce.d[c], d0, d1);
+        f2split(dn, n0, n1);
+        dn = f2pack((own.code & 4) ? d0 : n0, (own.code & 8) ? d1 : n1);
+      }
+      march_st<VEC>(dout, i + c * N, second, dn);
       float e0, e1;
       f2split(er, e0, e1);
       acc.max_lam(fabsf(e0));
