@@ -643,6 +643,7 @@ __global__ void k_param_contract(long long M, const double* dB, const double* mu
 namespace glemur {
 // Provided by glemur.cu.
 int ctx_recompute_stages(glemur_ctx* c, double dt, void* k6);
+bool ctx_two_pass(const glemur_ctx* c);
 int ctx_recompute_stages_saved(glemur_ctx* c, double dt, double* const* yS, double* const* BS,
                                double* const* GS);
 void ctx_dense_grid(const glemur_ctx* c, int most, int* grid, int* threads);
@@ -776,7 +777,7 @@ __global__ void k_adj_seed_boundary(AdjGeom g, const double* d, YSave ys, double
 }
 
 // The reverse step of an FP64 two-pass context, from the recompute's saved
-// data (kern_f64_vjp.cu).  BADARG for other contexts, with nothing done.
+// data (kern_f64_vjp.cu).
 int vjp_step_saved(glemur_ctx* c, const Adj& A, double dt, const double* lam_next, double* lam,
                    double* mu_B0) {
   double *yS[6] = {nullptr}, *BS[6], *GS[6];
@@ -861,10 +862,9 @@ template <typename T>
 int vjp_step_t(glemur_ctx* c, const Adj& A, double dt, const double* lam_next, double* lam,
                double* mu_B0) {
   const int N3 = 3 * A.N;
-  if (A.precision == GLEMUR_FP64) {
-    const int rs = vjp_step_saved(c, A, dt, lam_next, lam, mu_B0);
-    if (rs != GLEMUR_ERR_BADARG) return rs;
-  }
+  // (single-kernel FP64 contexts go on below, with no work queued for them here)
+  if (A.precision == GLEMUR_FP64 && ctx_two_pass(c))
+    return vjp_step_saved(c, A, dt, lam_next, lam, mu_B0);
   const int rc = ctx_recompute_stages(c, dt, A.ws + A.L.k6);
   if (rc) return rc;
   double* lamk_h[6];

@@ -904,15 +904,17 @@ int ctx_recompute_stages(glemur_ctx* c, double dt, void* k6) {
   return cuda_rc(e);
 }
 
-// The same recompute for FP64 two-pass contexts, keeping every stage's
+// FP64 mimetic stages in two passes, whose stage data a recompute can keep.
+bool ctx_two_pass(const glemur_ctx* c) { return c->o.curl == GLEMUR_CURL_MIMETIC && c->split; }
+
+// The same recompute for those contexts, keeping every stage's
 // data for the adjoint: stage s writes B into BS[s] (3N doubles) and its node
 // records into GS[s], and its next input y_{s+1} into yS[s+1] (3N doubles;
 // the caller has put the boundary positions in yS[1..5]); y_0 is the state
-// itself.  The last stage needs no velocity: its pass C is left out.  BADARG
-// for other contexts (the caller then recomputes stage data itself).
+// itself.  The last stage needs no velocity: its pass C is left out.
 int ctx_recompute_stages_saved(glemur_ctx* c, double dt, double* const* yS, double* const* BS,
                                double* const* GS) {
-  if (c->o.curl != GLEMUR_CURL_MIMETIC || !c->split) return GLEMUR_ERR_BADARG;
+  if (!ctx_two_pass(c)) return GLEMUR_ERR_BADARG;
   c->target_unbounded = 0;
   k_set_dt<<<1, 1, 0, c->s>>>(c->st, dt, 0);
   cudaError_t e = cudaGetLastError();
