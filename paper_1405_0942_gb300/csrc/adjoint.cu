@@ -644,6 +644,7 @@ namespace glemur {
 // Provided by glemur.cu.
 int ctx_recompute_stages(glemur_ctx* c, double dt, void* k6);
 bool ctx_two_pass(const glemur_ctx* c);
+void ctx_stage_buffers(const glemur_ctx* c, double* ys[2], double** Bb, double** Gb);
 int ctx_recompute_stages_saved(glemur_ctx* c, double dt, double* const* yS, double* const* BS,
                                double* const* GS);
 void ctx_dense_grid(const glemur_ctx* c, int most, int* grid, int* threads);
@@ -657,10 +658,20 @@ namespace {
 
 size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Adjoint workspace: k6 (storage type), FP64 stage input, B, 1/det, six
-// stage adjoints, the stage-input adjoint, the P and g adjoints, the
-// 1/det, centre-B, extra-B and velocity adjoints, mu (adjoint of B0s), the
-// xi partials and two small pointer tables.
+// Adjoint workspace: the P and g adjoints, the 1/det and centre-B adjoints,
+// the xi partials and two small pointer tables; then, in one place, since a
+// call uses either the one or the other:
+//   - k6 (storage type), FP64 stage input, B, 1/det, six stage adjoints, the
+//     stage-input adjoint, the extra-B and velocity adjoints and mu (adjoint
+//     of B0s): the loss gradients, and the reverse step that forms each
+//     stage's data itself;
+//   - what the reverse step of an FP64 two-pass context keeps of its forward
+//     recompute: y_1 .. y_3, B and the node records (G and 1/det G, whole
+//     warps of interior nodes) of stages 1 to 5.  y_4, y_5 and the last
+//     stage's B and records are the context's own buffers, and a stage's
+//     input adjoint takes its records' place once the stage is reversed.
+// 96 float64 values a node in FP64 (apart and without the context's buffers
+// they were 155; 384^3: 70.2 -> 43.5 GB).
 struct AdjLayout {
   size_t k6, y, Bb, rb, lamk, lamy, lamP, lamg, lamr, lamB, lamB2, lamu, mu, pv, pi, ptr,
       yS, BS, GS, total, fstride, gstride;
@@ -674,32 +685,32 @@ AdjLayout adj_layout(int nx, int ny, int nz, int precision) {
   AdjLayout L{};
   size_t o = 0;
   L.fstride = al(3 * N * 8);
+  L.lamP = o; o += al(9 * N * 8);
+  L.lamg = o; o += al(9 * N * 8);
+  L.lamr = o; o += al(N * 8);
+  L.lamB = o; o += L.fstride;
+  L.pv = o; o += al(kXiBlocks * 8 + 8);
+  L.pi = o; o += al(kXiBlocks * 4);
+  L.ptr = o; o += 256;
+  const size_t shared = o;
   L.k6 = o; o += al(3 * N * es);
   L.y = o; o += L.fstride;
   L.Bb = o; o += L.fstride;
   L.rb = o; o += al(N * 8);
   L.lamk = o; o += 6 * L.fstride;
   L.lamy = o; o += L.fstride;
-  L.lamP = o; o += al(9 * N * 8);
-  L.lamg = o; o += al(9 * N * 8);
-  L.lamr = o; o += al(N * 8);
-  L.lamB = o; o += L.fstride;
   L.lamB2 = o; o += L.fstride;
   L.lamu = o; o += L.fstride;
   L.mu = o; o += L.fstride;
-  L.pv = o; o += al(kXiBlocks * 8 + 8);
-  L.pi = o; o += al(kXiBlocks * 4);
-  L.ptr = o; o += 256;
-  // FP64: every stage's input (y_1..y_5), B and node records (G and 1/det G,
-  // whole warps of interior nodes), kept by the forward recompute so the
-  // reverse loop need not form them again
+  L.total = o;
   L.gstride = al(10 * (N + 31) * 8);
   if (precision == GLEMUR_FP64) {
-    L.yS = o; o += 5 * L.fstride;
-    L.BS = o; o += 6 * L.fstride;
-    L.GS = o; o += 6 * L.gstride;
+    o = shared;
+    L.yS = o; o += 3 * L.fstride;
+    L.BS = o; o += 5 * L.fstride;
+    L.GS = o; o += 5 * L.gstride;
+    if (o > L.total) L.total = o;
   }
-  L.total = o;
   return L;
 }
 
@@ -780,10 +791,12 @@ __global__ void k_adj_seed_boundary(AdjGeom g, const double* d, YSave ys, double
 // data (kern_f64_vjp.cu).
 int vjp_step_saved(glemur_ctx* c, const Adj& A, double dt, const double* lam_next, double* lam,
                    double* mu_B0) {
-  double *yS[6] = {nullptr}, *BS[6], *GS[6];
+  double *yS[6] = {nullptr}, *BS[6], *GS[6], *ys[2];
+  ctx_stage_buffers(c, ys, &BS[5], &GS[5]);
   YSave ysave;
-  for (int q = 1; q < 6; ++q) ysave.p[q - 1] = yS[q] = A.P(A.L.yS + (q - 1) * A.L.fstride);
-  for (int q = 0; q < 6; ++q) {
+  for (int q = 1; q < 6; ++q)
+    ysave.p[q - 1] = yS[q] = q < 4 ? A.P(A.L.yS + (q - 1) * A.L.fstride) : ys[q - 4];
+  for (int q = 0; q < 5; ++q) {
     BS[q] = A.P(A.L.BS + q * A.L.fstride);
     GS[q] = A.P(A.L.GS + q * A.L.gstride);
   }
@@ -801,7 +814,7 @@ int vjp_step_saved(glemur_ctx* c, const Adj& A, double dt, const double* lam_nex
   }
   v.B0s = (const double*)A.B0s;
   v.lam_next = lam_next;
-  for (int j = 0; j < 6; ++j) v.ly[j] = A.P(A.L.lamk + j * A.L.fstride);
+  for (int j = 0; j < 6; ++j) v.ly[j] = GS[j];  // its records are done with by then
   v.lamP = A.P(A.L.lamP);
   v.lamg = A.P(A.L.lamg);
   v.lamr = A.P(A.L.lamr);

@@ -907,6 +907,17 @@ int ctx_recompute_stages(glemur_ctx* c, double dt, void* k6) {
 // FP64 mimetic stages in two passes, whose stage data a recompute can keep.
 bool ctx_two_pass(const glemur_ctx* c) { return c->o.curl == GLEMUR_CURL_MIMETIC && c->split; }
 
+// Such a context's own stage inputs, B and node records: every attempt and
+// every call that runs a stage writes them anew (of the stage inputs the
+// interior: their boundary is the fixed boundary positions), so between such
+// calls another may use them.
+void ctx_stage_buffers(const glemur_ctx* c, double* ys[2], double** Bb, double** Gb) {
+  ys[0] = (double*)c->ys[0];
+  ys[1] = (double*)c->ys[1];
+  *Bb = c->Bb;
+  *Gb = c->Gb;
+}
+
 // The same recompute for those contexts, keeping every stage's
 // data for the adjoint: stage s writes B into BS[s] (3N doubles) and its node
 // records into GS[s], and its next input y_{s+1} into yS[s+1] (3N doubles;
