@@ -107,7 +107,8 @@ bool pdl_enabled() {
 // Eq. "time stepping" and the acceptance rule after each attempt (see
 // control.cuh), as a kernel of one CTA.
 // Its predecessor, the attempt's last stage, triggers it after its own wait,
-// so all earlier stages are complete when it starts.
+// so all earlier stages are complete when it starts.  It triggers its own
+// successor at once, which must not read ahead of its wait (see launch_pdl).
 __global__ void k_control(DevState* st, const double* part, int nb, int diag, double* dtlog) {
   pdl_trigger();
   __shared__ double sh[96];

@@ -102,16 +102,19 @@ struct StageArgs {
 // with launch_pdl: the next kernel of the stream may then be scheduled onto
 // SMs that the current one has left while its last CTAs still run.  Each
 // such kernel calls pdl_trigger() (its own successor may be scheduled once
-// all of its CTAs have started) and pdl_wait(): griddepcontrol.wait returns
-// once the preceding grids have completed and their memory operations are
-// visible.  Every path through such a kernel passes pdl_wait(), so
-// completion stays transitive along the stream.  Before it, a kernel reads
-// and writes nothing an earlier kernel of the stream touches, with one
-// exception: a stage after an attempt's first (its first pass counts as one)
-// and the step control trigger after their own pdl_wait(), so that when a
-// successor of theirs starts, everything before them is complete, and it may
-// read ahead of its wait what its immediate predecessor does not write (the
-// control state above all, which only the step control changes).
+// all of its CTAs have started and called it) and pdl_wait():
+// griddepcontrol.wait returns once the preceding grids have completed and
+// their memory operations are visible.  Every path through such a kernel
+// passes pdl_wait(), so completion stays transitive along the stream.  Before
+// it, a kernel reads and writes nothing an earlier kernel of the stream
+// touches, with one exception, which rests on this rule: every stage (both
+// its passes) triggers after its own pdl_wait().  So when what follows a stage
+// starts, everything before that stage is complete, and a stage after an
+// attempt's first, a pass after an attempt's first and the step control may
+// read ahead of their wait what the stage or pass before them does not write
+// (the control state but its flags, and the partials of the first stage's
+// diagnostics).  The step control triggers before its wait, so an attempt's
+// first stage or pass, like anything else that may follow it, waits first.
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
