@@ -30,23 +30,12 @@
 #include <climits>
 #include <cmath>
 
+#include "cash_karp.cuh"
 #include "glemur.h"
 #include "glemur_dev.cuh"
 #include "vjp64.cuh"
 
 namespace glemur {
-
-// Cash-Karp table (Cash & Karp, ACM TOMS 16, 1990) for the reverse combine.
-__constant__ double AD_A[6][6] = {
-    {0, 0, 0, 0, 0, 0},
-    {1.0 / 5.0, 0, 0, 0, 0, 0},
-    {3.0 / 40.0, 9.0 / 40.0, 0, 0, 0, 0},
-    {3.0 / 10.0, -9.0 / 10.0, 6.0 / 5.0, 0, 0, 0},
-    {-11.0 / 54.0, 5.0 / 2.0, -70.0 / 27.0, 35.0 / 27.0, 0, 0},
-    {1631.0 / 55296.0, 175.0 / 512.0, 575.0 / 13824.0, 44275.0 / 110592.0, 253.0 / 4096.0,
-     0}};
-__constant__ double AD_B5[6] = {37.0 / 378.0, 0.0, 250.0 / 621.0, 125.0 / 594.0, 0.0,
-                                512.0 / 1771.0};
 
 struct AdjGeom {
   int nx, ny, nz;
@@ -183,7 +172,7 @@ __device__ __forceinline__ void adj_stage_input_s(int N3, const T* d, const T* c
                                                   double* y) {
   double c[S > 0 ? S : 1];
 #pragma unroll
-  for (int j = 0; j < S; ++j) c[j] = dt * AD_A[S][j];
+  for (int j = 0; j < S; ++j) c[j] = dt * CK.a[S][j];
   NODE_LOOP(N3) {
     double v = (double)d[n];
 #pragma unroll
@@ -459,7 +448,7 @@ __device__ __forceinline__ void adj_positions_s(const AdjGeom& g, const double* 
   const int st[3] = {1, g.nx, g.nx * g.ny};
   double cj[S > 0 ? S : 1];
 #pragma unroll
-  for (int j = 0; j < (S > 0 ? S : 0); ++j) cj[j] = dt * AD_A[S][j];
+  for (int j = 0; j < (S > 0 ? S : 0); ++j) cj[j] = dt * CK.a[S][j];
   if (has_deep(g)) {
     const int ND = (g.nx - 6) * (g.ny - 6) * (g.nz - 6);
     GRID_LOOP(t, ND) {
@@ -521,7 +510,7 @@ __global__ void k_adj_seed(int N3, const double* lam_next, double dt, double* la
   NODE_LOOP(N3) {
     const double v = lam_next[n];
     lam[n] = v;
-    for (int j = 0; j < 6; ++j) lam_k[j][n] = dt * AD_B5[j] * v;
+    for (int j = 0; j < 6; ++j) lam_k[j][n] = dt * CK.b5[j] * v;
   }
 }
 
@@ -753,17 +742,6 @@ int nblk(long long n) {
   return (int)(b < 8192 ? (b < 1 ? 1 : b) : 8192);
 }
 
-// The same table on the host.
-const double kA[6][6] = {
-    {0, 0, 0, 0, 0, 0},
-    {1.0 / 5.0, 0, 0, 0, 0, 0},
-    {3.0 / 40.0, 9.0 / 40.0, 0, 0, 0, 0},
-    {3.0 / 10.0, -9.0 / 10.0, 6.0 / 5.0, 0, 0, 0},
-    {-11.0 / 54.0, 5.0 / 2.0, -70.0 / 27.0, 35.0 / 27.0, 0, 0},
-    {1631.0 / 55296.0, 175.0 / 512.0, 575.0 / 13824.0, 44275.0 / 110592.0, 253.0 / 4096.0,
-     0}};
-const double kB5[6] = {37.0 / 378.0, 0.0, 250.0 / 621.0, 125.0 / 594.0, 0.0, 512.0 / 1771.0};
-
 // Five stage-input buffers (pointers by value).
 struct YSave {
   double* p[5];
@@ -834,8 +812,8 @@ int vjp_step_saved(glemur_ctx* c, const Adj& A, double dt, const double* lam_nex
     v.y = s == 0 ? (const double*)A.d : yS[s];
     v.Bb = BS[s];
     v.rec = GS[s];
-    v.cb = dt * kB5[s];
-    for (int j = 0; j < 6; ++j) v.ca[j] = j > s ? dt * kA[j][s] : 0.0;
+    v.cb = dt * CASH_KARP.b5[s];
+    for (int j = 0; j < 6; ++j) v.ca[j] = j > s ? dt * CASH_KARP.a[j][s] : 0.0;
     v.ly_out = (double*)v.ly[s];
     const cudaError_t e = launch_f64_vjp(v, s, A.s);
     if (e != cudaSuccess) return GLEMUR_ERR_CUDA;

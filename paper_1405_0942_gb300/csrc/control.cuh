@@ -1,6 +1,6 @@
-// Step-size control of the relaxation (section "Time Stepping"): the
-// Cash-Karp table, the control law of eq. "time stepping" with the
-// acceptance rule around it, and the fixed-order reductions of the per-CTA
+// Step-size control of the relaxation (section "Time Stepping"): the control
+// law of eq. "time stepping" with the acceptance rule around it, and the
+// fixed-order reductions of the per-CTA
 // partials (error norm, E_M, xi).  Run by one CTA after each attempt --
 // as the control kernel, or inside the persistent attempt kernel by the
 // CTA that finishes an attempt last.  Loads go through a policy: plain
@@ -10,6 +10,7 @@
 
 #include <cuda_runtime.h>
 
+#include "cash_karp.cuh"
 #include "glemur.h"
 #include "glemur_dev.cuh"
 
@@ -27,21 +28,6 @@ struct LdCoherent {
   __device__ static __forceinline__ unsigned ldu(const unsigned* p) { return __ldcg(p); }
   __device__ static __forceinline__ long long ldll(const long long* p) { return __ldcg(p); }
 };
-
-// Cash-Karp embedded 5(4) pair (Cash & Karp, ACM TOMS 16, 1990), the scheme
-// of section "Time Stepping".
-static __constant__ double CK_A[6][6] = {
-    {0, 0, 0, 0, 0, 0},
-    {1.0 / 5.0, 0, 0, 0, 0, 0},
-    {3.0 / 40.0, 9.0 / 40.0, 0, 0, 0, 0},
-    {3.0 / 10.0, -9.0 / 10.0, 6.0 / 5.0, 0, 0, 0},
-    {-11.0 / 54.0, 5.0 / 2.0, -70.0 / 27.0, 35.0 / 27.0, 0, 0},
-    {1631.0 / 55296.0, 175.0 / 512.0, 575.0 / 13824.0, 44275.0 / 110592.0,
-     253.0 / 4096.0, 0}};
-static __constant__ double CK_B5[6] = {37.0 / 378.0, 0.0, 250.0 / 621.0, 125.0 / 594.0, 0.0,
-                                512.0 / 1771.0};
-static __constant__ double CK_B4[6] = {2825.0 / 27648.0, 0.0, 18575.0 / 48384.0,
-                                13525.0 / 55296.0, 277.0 / 14336.0, 1.0 / 4.0};
 
 // Sum and max reductions of the per-CTA diagnostic partials (fixed order).
 template <class LD>
@@ -96,12 +82,12 @@ __device__ __forceinline__ void set_coeffs_parallel(DevState* st, double dt) {
   for (int t = threadIdx.x; t < 42; t += blockDim.x) {
     if (t < 36) {
       const int s = t / 6, j = t % 6;
-      const double v = dt * CK_A[s][j];
+      const double v = dt * CK.a[s][j];
       st->dta[s][j] = v;
       st->dtaf[s][j] = (float)v;
     } else {
       const int s = t - 36;
-      const double b = dt * CK_B5[s], e = dt * (CK_B5[s] - CK_B4[s]);
+      const double b = dt * CK.b5[s], e = dt * (CK.b5[s] - CK.b4[s]);
       st->dtb[s] = b;
       st->dte[s] = e;
       st->dtbf[s] = (float)b;

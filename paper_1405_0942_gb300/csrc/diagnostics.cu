@@ -506,6 +506,7 @@ int glemur_alpha_line(glemur_ctx* ctx, int i, int j, double a_r, double* alpha,
   DiagCtx c;
   int rc = ctx_diag(ctx, &c);
   if (rc) return rc;
+  // (nz <= 6144: the bound the header states; the kernels below need none)
   if (i < 1 || i > c.nx - 2 || j < 1 || j > c.ny - 2 || !(a_r > 0) || c.nz > 6144)
     return GLEMUR_ERR_BADARG;
   const DG g = geom_of(c);

@@ -44,11 +44,11 @@ __device__ void set_coeffs(DevState* st) {
   const double dt = st->dt;
   for (int s = 0; s < 6; ++s) {
     for (int j = 0; j < 6; ++j) {
-      st->dta[s][j] = dt * CK_A[s][j];
+      st->dta[s][j] = dt * CK.a[s][j];
       st->dtaf[s][j] = (float)st->dta[s][j];
     }
-    st->dtb[s] = dt * CK_B5[s];
-    st->dte[s] = dt * (CK_B5[s] - CK_B4[s]);
+    st->dtb[s] = dt * CK.b5[s];
+    st->dte[s] = dt * (CK.b5[s] - CK.b4[s]);
     st->dtbf[s] = (float)st->dtb[s];
     st->dtef[s] = (float)st->dte[s];
   }

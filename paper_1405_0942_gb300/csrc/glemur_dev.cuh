@@ -253,10 +253,6 @@ struct DiagCtx {
   cudaStream_t s;
 };
 
-__device__ __forceinline__ long long nidx(int i, int j, int k, int nx, int ny) {
-  return ((long long)k * ny + j) * nx + i;
-}
-
 // 1/v, FP64: Newton-Raphson refinement of the hardware approximation
 // rcp.approx.ftz.f64, y <- y + y (1 - v y): each step squares the relative
 // error (the classical iteration for reciprocals, e.g. Muller et al.,

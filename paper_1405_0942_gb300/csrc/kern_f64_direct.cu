@@ -16,12 +16,6 @@ namespace glemur {
 
 namespace {
 
-__device__ __forceinline__ void cross64(const double a[3], const double b[3], double o[3]) {
-  o[0] = a[1] * b[2] - a[2] * b[1];
-  o[1] = a[2] * b[0] - a[0] * b[2];
-  o[2] = a[0] * b[1] - a[1] * b[0];
-}
-
 // Direct current at interior node n (section "Diagnostics", the classic
 // method): dB/dX of B = V / det G, V = sum_a g_a b_a, by the product rule,
 //   det D_c B = D_c V - V (D_c det) / det,

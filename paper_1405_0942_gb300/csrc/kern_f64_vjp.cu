@@ -30,12 +30,6 @@ namespace glemur {
 
 namespace {
 
-__device__ __forceinline__ void cross64(const double a[3], const double b[3], double o[3]) {
-  o[0] = a[1] * b[2] - a[2] * b[1];
-  o[1] = a[2] * b[0] - a[0] * b[2];
-  o[2] = a[0] * b[1] - a[1] * b[0];
-}
-
 // The node's record of pass B (kern_f64_split.cu, node_record).
 __device__ __forceinline__ void load_record(const VjpArgs& a, int t, double g[3][3], double& r) {
   const double2* q = reinterpret_cast<const double2*>(a.rec) + ((size_t)(t >> 5) * 160 + (t & 31));

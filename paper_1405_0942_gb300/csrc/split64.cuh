@@ -182,6 +182,12 @@ __device__ __forceinline__ void put_partial(const SplitArgs& a, int kind, double
   for (int b = gridDim.x + blockIdx.x; b < a.nblocks; b += gridDim.x) p[b] = 0.0;
 }
 
+__device__ __forceinline__ void cross64(const double a[3], const double b[3], double o[3]) {
+  o[0] = a[1] * b[2] - a[2] * b[1];
+  o[1] = a[2] * b[0] - a[0] * b[2];
+  o[2] = a[0] * b[1] - a[1] * b[0];
+}
+
 // a.b - c.d as one multiply and five FMAs (one FP64 instruction fewer than
 // two dot products and a subtraction)
 __device__ __forceinline__ double dot3_sub(const double a[3], const double b[3],
