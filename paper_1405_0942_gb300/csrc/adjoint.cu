@@ -1021,8 +1021,10 @@ int glemur_adjoint_segment(glemur_ctx* c, const double* x0, const double* dts, i
   for (long long q = nseg - 1; q >= 0; --q) {
     const int start = (int)(q * every), end = start + every < n ? start + every : n;
     // the states between its steps: the last segment's are kept already, and
-    // no segment's last step is needed (64^3, four steps, a checkpoint every
-    // two: one step repeated instead of four, 7.30 -> 6.28 ms)
+    // no segment's last step is needed, so (nseg - 1)(every - 1) of n steps
+    // are repeated instead of all (64^3, four steps, a checkpoint every two:
+    // one, 7.30 -> 6.28 ms; 500 steps, one every 50: 441, about 2 % of the
+    // gradient's time; none where n <= every)
     if (start != last && end - start > 1) {
       if ((rc = glemur_set_state(c, ckpt(q)))) return rc;
       for (int i = start; i + 1 < end; ++i) {
