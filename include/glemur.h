@@ -157,7 +157,8 @@ size_t glemur_workspace_bytes(int nx, int ny, int nz, int precision);
  *                         recomputation) instead of the two-pass stages
  *   GLEMUR_KZ=k           z-planes per CTA of the stage kernels instead of
  *                         the cost model's choice (more where k are too few
- *                         for a launch: 65535 slabs at most)
+ *                         for a launch: 65535 slabs at most), and the mixed
+ *                         mimetic stages on the 64-wide march for any nx
  *   GLEMUR_PERSIST=1      FP64 two-pass stages, line-tied, loop currents:
  *                         whole attempts (twelve passes and the control) in
  *                         one persistent cooperative launch with per-plane

@@ -22,14 +22,17 @@ cudaError_t launch_f64_mimetic(const StageArgs<double>& a, int stage, dim3 grid,
 cudaError_t launch_f64_direct(const SplitArgs& a, int stage, cudaStream_t s);
 cudaError_t launch_f32_mimetic(const StageArgs<float>& a, const TmaMaps* maps, int stage,
                                dim3 grid, cudaStream_t s);
+cudaError_t launch_f32_narrow(const StageArgs<float>& a, int stage, dim3 grid, cudaStream_t s);
 cudaError_t launch_f32_direct(const StageArgs<float>& a, int stage, dim3 grid, cudaStream_t s);
 cudaError_t prepare_f64_mimetic();
 cudaError_t prepare_f32_mimetic();
+cudaError_t prepare_f32_narrow();
 cudaError_t prepare_f32_direct();
 int ctas_per_sm_f64_mimetic();
 int ctas_per_sm_f32_mimetic(bool tma);
 int tile_rows_f32_mimetic();
 int tile_cols_f32_mimetic();
+int ctas_per_sm_f32_narrow();
 int ctas_per_sm_f32_direct();
 
 cudaError_t launch_f64_split(const SplitArgs& a, int stage, cudaStream_t s, int curl,
@@ -299,7 +302,8 @@ struct glemur_ctx {
   DevState* st;
   double* dtlog;    // ring of GLEMUR_DT_LOG accepted step sizes
   int split;                             // FP64 mimetic stages in two passes
-  int tma;                               // mixed mimetic stages with TMA tiles
+  int tma;                               // mixed mimetic march with TMA tiles
+  int narrow;                            // mixed mimetic stages on 32-wide tiles
   int early;                             // stage grids that leave room for the next
   int tma_test;                          // test hook: unsatisfiable tile wait
   TmaMaps maps;                          // their tensor maps
@@ -506,13 +510,13 @@ int kz_from_env(int nz) {
   return kz < 1 ? 0 : (kz > nz ? nz : (kz < least ? least : kz));
 }
 
-// Planes per CTA along z of the fused FP64 and the mixed direct stage kernels.
+// Planes per CTA along z of the stage kernels on 32-wide tiles.
 // Cost model: the time of the busiest SM, in units of one B plane (a CTA of
 // kz planes computes kz + 2 B planes).  FP64 stages are bound by the SM's
 // FP64 pipe, which co-resident CTAs share, so an SM's time is its CTA count x
 // (kz + 2); the FP32 stages are latency-bound, so up to `per_sm` co-resident
 // CTAs overlap and the time is waves x (kz + 2).
-int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe) {
+int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe, double* cost_out = nullptr) {
   if (const int kz = kz_from_env(nz)) return kz;
   if (nsm < 1) nsm = 1;
   if (per_sm < 1) per_sm = 1;
@@ -528,10 +532,11 @@ int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe) {
       best = kz;
     }
   }
+  if (cost_out) *cost_out = best_cost;
   return best;
 }
 
-// Planes per CTA along z of the mixed mimetic stage: the shortest schedule
+// Planes per CTA along z of the mixed mimetic march: the shortest schedule
 // of its CTAs on the SMs' slots.  A CTA of kz planes runs kz + 2 iterations
 // and its prologue takes about half of one; the last slab's CTAs, of the
 // remaining planes, are shorter (one halo plane less) and start last.  They
@@ -544,7 +549,7 @@ int choose_kz(int nz, int gxy, int nsm, int per_sm, bool shared_pipe) {
 // (384^3: kz = 28, 36, 48 take 4.89, 4.85, 4.91 ms, 192 takes 9 % more than
 // 32), hence the limit of 40 -- more where 40 planes each are more slabs than
 // a launch counts along z (3 x 3 x 2621403).
-int choose_kz_march(int nz, int gxy, int nsm, int per_sm) {
+int choose_kz_march(int nz, int gxy, int nsm, int per_sm, double* cost_out) {
   if (const int kz = kz_from_env(nz)) return kz;
   if (nsm < 1) nsm = 1;
   if (per_sm < 1) per_sm = 1;
@@ -575,7 +580,27 @@ int choose_kz_march(int nz, int gxy, int nsm, int per_sm) {
       best = kz;
     }
   }
+  *cost_out = best_cost;
   return best;
+}
+
+// Whether the mixed mimetic stages run on 32-wide tiles, one node per thread
+// (kern_f32_narrow.cu), instead of the march's 64-wide ones.  Both schedules'
+// costs are in iterations, and an iteration of the one takes as long as one of
+// the march with plain copies (17.5 and 18 us an attempt; with TMA 13.6, and 8
+// once), so the ratio of the costs is that of the times where both fill the
+// chip.  It is below 1 where an x row takes an odd number of 32-wide tiles, so
+// that half of the march's last tile is idle, and few (the march's attempt and
+// this one's: 24 x 200 x 150 247, 203 us; 70 x 66 x 61 119, 110; 90 x 31 x 200
+// 154, 145; 130 x 120 x 60 229, 215; 3 x 400 x 400 1004, 727).  Of 320 grids
+// with rows of 3 to 321 nodes none selected so was faster on the march, and
+// none of the others slower by more than 4 %.  With TMA only rows of one
+// 32-wide tile lose (cost ratios 0.71 to 0.78: 24 x 200 x 150 220, 203; 20 x
+// 1000 x 20 162, 149; at 0.89 24 x 64 x 64 73, 71 and 32 x 64 x 64 71, 73).  A
+// march of one CTA per SM at most has shorter iterations and stays (12^3 40
+// against 47 us, 33^3 55 against 61).
+bool choose_narrow(double cost_narrow, double cost_march, long long march_ctas, int nsm, bool tma) {
+  return march_ctas > nsm && cost_narrow < (tma ? 0.8 : 1.0) * cost_march;
 }
 
 // Grid of a dense FP64 pass over the interior nodes and, for pass B, the
@@ -683,6 +708,7 @@ cudaError_t launch_stage(const glemur_ctx* c, int curl, int stage, int diag, int
       a.nblocks = c->nblocks_direct;
       return launch_f32_direct(a, stage, g, c->s);
     }
+    if (c->narrow) return launch_f32_narrow(a, stage, g, c->s);
     return launch_f32_mimetic(a, c->tma ? &c->maps : nullptr, stage, g, c->s);
   }
   if (curl == GLEMUR_CURL_DIRECT) {
@@ -1097,6 +1123,7 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   const char* tt = getenv("GLEMUR_TEST_TMA_TIMEOUT");
   c->tma_test = tt && (atoi(tt) == 1 || atoi(tt) == 2) ? atoi(tt) : 0;
   if (e == cudaSuccess && setup_tma(c)) c->tma = 1;
+  if (e == cudaSuccess && mixed) e = prepare_f32_narrow();
   if (e == cudaSuccess && mixed) e = prepare_f32_direct();
   if (e != cudaSuccess) {
     delete c;
@@ -1106,18 +1133,33 @@ int glemur_init_grid(glemur_ctx** out, int nx, int ny, int nz, const double lo[3
   c->dense_c = dense_shape(c, false, o.curl == GLEMUR_CURL_NNN ? DENSE_T2 : DENSE_T);
   c->dense_direct = dense_shape(c, false, DENSE_T2);
   const int gx = (nx + TX - 1) / TX, gy = (ny + TY - 1) / TY;
-  const int twm = mixed ? tile_cols_f32_mimetic() : TX;
-  const int thm = mixed ? tile_rows_f32_mimetic() : TY;
-  const int gxm = (nx + twm - 1) / twm, gym = (ny + thm - 1) / thm;
-  const int pm = mixed ? ctas_per_sm_f32_mimetic(c->tma != 0) : ctas_per_sm_f64_mimetic();
-  c->kz = mixed ? choose_kz_march(nz, gxm * gym, c->nsm, pm)
-                : choose_kz(nz, gxm * gym, c->nsm, pm, true);
-  c->grid = dim3(gxm, gym, (nz + c->kz - 1) / c->kz);
-  c->nblocks = gxm * gym * (int)c->grid.z;
-  // a grid that leaves room beside it for the next stage's lets that one
-  // start its prologue meanwhile (48^3: 59.6 -> 58.7 us an attempt); a larger
-  // one's waiting CTAs would hold the slots its own still need
-  c->early = mixed && 2LL * c->nblocks <= (long long)pm * c->nsm;
+  c->narrow = 0;
+  if (mixed) {
+    const int gxm = (nx + tile_cols_f32_mimetic() - 1) / tile_cols_f32_mimetic();
+    const int gym = (ny + tile_rows_f32_mimetic() - 1) / tile_rows_f32_mimetic();
+    const int pm = ctas_per_sm_f32_mimetic(c->tma != 0);
+    double cost_m = 0.0, cost_n = 0.0;  // (both 0 where GLEMUR_KZ gives the planes)
+    c->kz = choose_kz_march(nz, gxm * gym, c->nsm, pm, &cost_m);
+    const int kzn = choose_kz(nz, gx * gy, c->nsm, ctas_per_sm_f32_narrow(), false, &cost_n);
+    c->grid = dim3(gxm, gym, (nz + c->kz - 1) / c->kz);
+    c->nblocks = gxm * gym * (int)c->grid.z;
+    if (choose_narrow(cost_n, cost_m, c->nblocks, c->nsm, c->tma != 0)) {
+      c->narrow = 1;
+      c->tma = 0;
+      c->kz = kzn;
+      c->grid = dim3(gx, gy, (nz + kzn - 1) / kzn);
+      c->nblocks = gx * gy * (int)c->grid.z;
+    }
+    // a march that leaves room beside it for the next stage's lets that one
+    // start its prologue meanwhile (48^3: 59.6 -> 58.7 us an attempt); a larger
+    // one's waiting CTAs would hold the slots its own still need
+    c->early = 2LL * c->nblocks <= (long long)pm * c->nsm;
+  } else {
+    c->early = 0;
+    c->kz = choose_kz(nz, gx * gy, c->nsm, ctas_per_sm_f64_mimetic(), true);
+    c->grid = dim3(gx, gy, (nz + c->kz - 1) / c->kz);
+    c->nblocks = gx * gy * (int)c->grid.z;
+  }
   if (c->split) {
     // one CTA per SM; the partials' stride is the larger grid
     c->nblocks = c->dense_b.grid > c->dense_c.grid ? c->dense_b.grid : c->dense_c.grid;
