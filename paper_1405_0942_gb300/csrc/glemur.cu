@@ -161,26 +161,36 @@ __device__ __forceinline__ double widen(float v) {
 // Conversions of whole fields: a thread takes a node of the (x, y) plane and
 // up to CONV_PLANES planes of it, so that the node labels (a conversion and
 // an FMA on the FP64 pipe each) cost a few of its instructions per column,
-// with CONV_BATCH planes' loads in flight.  Small grids take fewer planes per
-// CTA, so that every SM has one (16^3 with 8 planes, two CTAs: a call of
-// set_x takes 13.8 us, with one plane 11.8).
+// with BATCH planes' loads in flight.  Small grids take fewer planes per
+// thread, so that every SM has a CTA, one plane at a time in a shorter code
+// (a launch starts on a cold instruction cache); of planes of fewer nodes than
+// a CTA's threads it takes `rows` at a time, adjacent ones, so that a warp's
+// accesses stay contiguous (3 x 3 x 400000 mixed, one plane at a time: get_x
+// 174 us, so 33).
 constexpr int CONV_T = 256, CONV_PLANES = 8, CONV_BATCH = 4;
 struct Column {
-  int p, k0, k1;  // node of the plane, planes [k0, k1)
+  int p;        // node of the plane (nx ny or more: none)
+  int kz, kc;   // the CTA's first plane, the thread's: kc, kc + rows, ..
 };
-__device__ __forceinline__ Column conv_column(const GridGeom& g, int planes) {
-  const int cb = (g.nx * g.ny + CONV_T - 1) / CONV_T;
-  const int k0 = (int)(blockIdx.x / cb) * planes;
-  return {(int)(blockIdx.x % cb) * CONV_T + (int)threadIdx.x, k0, min(k0 + planes, g.nz)};
+__device__ __forceinline__ Column conv_column(const GridGeom& g, int planes, int rows) {
+  const int nxy = g.nx * g.ny, t = threadIdx.x, b = blockIdx.x;
+  if (rows > 1) {
+    const int r = t / nxy, kz = b * rows * planes;
+    return {r < rows ? t - r * nxy : nxy, kz, kz + r};
+  }
+  const int cb = (nxy + CONV_T - 1) / CONV_T, q = b / cb;
+  return {(b - q * cb) * CONV_T + t, q * planes, q * planes};
 }
 struct ConvGrid {
-  int planes, blocks;
+  int planes, rows, blocks;
 };
 ConvGrid conv_grid(int nx, int ny, int nz, int nsm) {
-  const int cb = (nx * ny + CONV_T - 1) / CONV_T;
+  const int nxy = nx * ny, cb = (nxy + CONV_T - 1) / CONV_T;
+  const int rows = cb > 1 ? 1 : CONV_T / nxy;
   int planes = CONV_PLANES;
-  while (planes > 1 && (long long)cb * ((nz + planes - 1) / planes) < nsm) planes /= 2;
-  return {planes, cb * ((nz + planes - 1) / planes)};
+  auto blocks = [&] { return cb * ((nz + planes * rows - 1) / (planes * rows)); };
+  while (planes > 1 && blocks() < nsm) planes /= 2;
+  return {planes, rows, blocks()};
 }
 
 // d = x - X into the current displacements, and into the boundary nodes of
@@ -188,39 +198,44 @@ ConvGrid conv_grid(int nx, int ny, int nz, int nsm) {
 // every interior node of these before they read it, and no boundary node.
 // Of 72 B per node of a mixed field that leaves the 36 of x and d, and of 12
 // FP64 instructions 3 (a call at 384^3: 1.28 -> 0.42 ms, HBM's share 0.30;
-// 256^3 in FP64 324 -> 160 us).  Grids hold fewer than 2^31 / 3 nodes, so
-// 32-bit indices suffice.
-template <typename T>
-__global__ void __launch_bounds__(CONV_T) k_set_x(GridGeom g, int planes,
+// 256^3 in FP64 324 -> 160 us).  `all`: into every node of them, where the
+// boundary is a third of the grid or more and its scattered nodes would leave
+// most 32-byte sectors in parts (8 x 8 x 100000 FP64 197 -> 129 us; 20 x 20 x
+// 1000, of which it is a fifth, 15 against 19).  Grids hold fewer than 2^31 /
+// 3 nodes, so 32-bit indices suffice.
+template <typename T, int BATCH>
+__global__ void __launch_bounds__(CONV_T) k_set_x(GridGeom g, int planes, int rows, bool all,
                                                   const double* __restrict__ x, T* d0, T* d1, T* y0, T* y1) {
-  __shared__ double Z[CONV_PLANES];
-  const Column w = conv_column(g, planes);
+  __shared__ double Z[CONV_T];
+  const Column w = conv_column(g, planes, rows);
   const int nxy = g.nx * g.ny, N = nxy * g.nz;
   // periodic in z: a ghost plane takes its partner's displacement (the
   // ghost's position is the partner's shifted by the period)
   auto source = [&](int k) {
     return g.periodic && k == 0 ? g.nz - 2 : (g.periodic && k == g.nz - 1 ? 1 : k);
   };
-  if (threadIdx.x < CONV_PLANES) Z[threadIdx.x] = label(g, 2, source(w.k0 + threadIdx.x));
+  if (threadIdx.x < planes * rows) Z[threadIdx.x] = label(g, 2, source(w.kz + threadIdx.x));
   __syncthreads();
   if (w.p >= nxy) return;
-  const int i = w.p % g.nx, j = w.p / g.nx;
+  const int j = w.p / g.nx, i = w.p - j * g.nx;
   const double X = label(g, 0, i), Y = label(g, 1, j);
-  const bool side = i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1;
-  for (int kb = w.k0; kb < w.k1; kb += CONV_BATCH) {
-    double v[CONV_BATCH][3];
+  const bool side = all || i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1;
+  for (int m = 0; m < planes; m += BATCH) {
+    double v[BATCH][3];
 #pragma unroll
-    for (int q = 0; q < CONV_BATCH; ++q)
-      if (kb + q < w.k1) {
-        const int n = source(kb + q) * nxy + w.p;
+    for (int q = 0; q < BATCH; ++q) {
+      const int k = w.kc + (m + q) * rows;
+      if (k < g.nz) {
+        const int n = source(k) * nxy + w.p;
         for (int c = 0; c < 3; ++c) v[q][c] = x[c * N + n];
       }
+    }
 #pragma unroll
-    for (int q = 0; q < CONV_BATCH; ++q) {
-      const int k = kb + q;
-      if (k >= w.k1) break;
+    for (int q = 0; q < BATCH; ++q) {
+      const int k = w.kc + (m + q) * rows;
+      if (k >= g.nz) return;
       const int n = k * nxy + w.p;
-      const double L[3] = {X, Y, Z[k - w.k0]};
+      const double L[3] = {X, Y, Z[k - w.kz]};
       T d[3];
       for (int c = 0; c < 3; ++c) {
         narrow(v[q][c] - L[c], d[c]);
@@ -232,26 +247,36 @@ __global__ void __launch_bounds__(CONV_T) k_set_x(GridGeom g, int planes,
   }
 }
 
-// x = X + d (384^3 mixed: 1.25 -> 0.45 ms; 256^3 in FP64 287 -> 148 us)
-template <typename T>
-__global__ void __launch_bounds__(CONV_T) k_get_x(GridGeom g, int planes,
+// x = X + d (384^3 mixed: 1.25 -> 0.39 ms; 256^3 in FP64 287 -> 150 us)
+template <typename T, int BATCH>
+__global__ void __launch_bounds__(CONV_T) k_get_x(GridGeom g, int planes, int rows,
                                                   const T* const* dbuf, const DevState* st,
                                                   double* __restrict__ x) {
-  __shared__ double Z[CONV_PLANES];
-  const Column w = conv_column(g, planes);
+  __shared__ double Z[CONV_T];
+  const Column w = conv_column(g, planes, rows);
   const int nxy = g.nx * g.ny, N = nxy * g.nz;
   const T* __restrict__ d = dbuf[st->cur];
-  if (threadIdx.x < CONV_PLANES) Z[threadIdx.x] = label(g, 2, w.k0 + threadIdx.x);
+  if (threadIdx.x < planes * rows) Z[threadIdx.x] = label(g, 2, w.kz + threadIdx.x);
   __syncthreads();
   if (w.p >= nxy) return;
-  const double X = label(g, 0, w.p % g.nx), Y = label(g, 1, w.p / g.nx);
-#pragma unroll CONV_PLANES
-  for (int q = 0; q < CONV_PLANES; ++q) {
-    const int k = w.k0 + q;
-    if (k >= w.k1) break;
-    const int n = k * nxy + w.p;
-    const double L[3] = {X, Y, Z[q]};
-    for (int c = 0; c < 3; ++c) x[c * N + n] = L[c] + widen(d[c * N + n]);
+  const int j = w.p / g.nx;
+  const double X = label(g, 0, w.p - j * g.nx), Y = label(g, 1, j);
+  for (int m = 0; m < planes; m += BATCH) {
+    T v[BATCH][3];
+#pragma unroll
+    for (int q = 0; q < BATCH; ++q) {
+      const int k = w.kc + (m + q) * rows;
+      if (k < g.nz)
+        for (int c = 0; c < 3; ++c) v[q][c] = d[c * N + k * nxy + w.p];
+    }
+#pragma unroll
+    for (int q = 0; q < BATCH; ++q) {
+      const int k = w.kc + (m + q) * rows;
+      if (k >= g.nz) return;
+      const int n = k * nxy + w.p;
+      const double L[3] = {X, Y, Z[k - w.kz]};
+      for (int c = 0; c < 3; ++c) x[c * N + n] = L[c] + widen(v[q][c]);
+    }
   }
 }
 
@@ -1207,14 +1232,18 @@ int glemur_set_x(glemur_ctx* c, const double* x, int mem) {
   int rc = stage_in(c, x, mem, &src);
   if (rc) return rc;
   const ConvGrid cg = conv_grid(c->nx, c->ny, c->nz, c->nsm);
+  auto set = [&](auto kernel, auto* d0, auto* d1, auto* y0, auto* y1) {
+    const long long inner = (long long)(c->nx - 2) * (c->ny - 2) * (c->nz - 2);
+    kernel<<<cg.blocks, CONV_T, 0, c->s>>>(geom(c), cg.planes, cg.rows, 3 * inner < 2 * c->N, src,
+                                           d0, d1, y0, y1);
+  };
+  const bool batch = cg.planes >= CONV_BATCH;
   if (c->o.precision == GLEMUR_MIXED)
-    k_set_x<float><<<cg.blocks, CONV_T, 0, c->s>>>(
-        geom(c), cg.planes, src, (float*)c->dbuf[0], (float*)c->dbuf[1], (float*)c->ys[0],
-        (float*)c->ys[1]);
+    set(batch ? k_set_x<float, CONV_BATCH> : k_set_x<float, 1>, (float*)c->dbuf[0],
+        (float*)c->dbuf[1], (float*)c->ys[0], (float*)c->ys[1]);
   else
-    k_set_x<double><<<cg.blocks, CONV_T, 0, c->s>>>(
-        geom(c), cg.planes, src, (double*)c->dbuf[0], (double*)c->dbuf[1], (double*)c->ys[0],
-        (double*)c->ys[1]);
+    set(batch ? k_set_x<double, CONV_BATCH> : k_set_x<double, 1>, (double*)c->dbuf[0],
+        (double*)c->dbuf[1], (double*)c->ys[0], (double*)c->ys[1]);
   rc = cuda_rc(cudaGetLastError());
   if (rc) return rc;
   return reset_state(c);  // k_set_x also seeded the stage inputs
@@ -1263,12 +1292,13 @@ int glemur_get_x(glemur_ctx* c, double* x, int mem) {
   if (!c || !x || (mem != GLEMUR_MEM_DEVICE && mem != GLEMUR_MEM_HOST)) return GLEMUR_ERR_BADARG;
   double* dst = out_target(c, x, mem);
   const ConvGrid cg = conv_grid(c->nx, c->ny, c->nz, c->nsm);
+  const bool batch = cg.planes >= CONV_BATCH;
   if (c->o.precision == GLEMUR_MIXED)
-    k_get_x<float><<<cg.blocks, CONV_T, 0, c->s>>>(
-        geom(c), cg.planes, (const float* const*)c->dbuf_dev, c->st, dst);
+    (batch ? k_get_x<float, CONV_BATCH> : k_get_x<float, 1>)<<<cg.blocks, CONV_T, 0, c->s>>>(
+        geom(c), cg.planes, cg.rows, (const float* const*)c->dbuf_dev, c->st, dst);
   else
-    k_get_x<double><<<cg.blocks, CONV_T, 0, c->s>>>(
-        geom(c), cg.planes, (const double* const*)c->dbuf_dev, c->st, dst);
+    (batch ? k_get_x<double, CONV_BATCH> : k_get_x<double, 1>)<<<cg.blocks, CONV_T, 0, c->s>>>(
+        geom(c), cg.planes, cg.rows, (const double* const*)c->dbuf_dev, c->st, dst);
   int rc = cuda_rc(cudaGetLastError());
   if (rc) return rc;
   return stage_out(c, x, dst, mem);

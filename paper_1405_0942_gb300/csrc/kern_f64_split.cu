@@ -44,9 +44,8 @@ __device__ __forceinline__ double2* node_record(const SplitArgs& a, int t) {
 
 // det G, 1/det G and B = G B0s / det G at node n from its columns (eq. "B
 // transformation"); B stored at node nw (n itself, or a periodic ghost node
-// that carries n's B), with G: the
-// differences and 1/det G interleaved for pass C (interior nodes).  Returns
-// the node's energy term zeta |B|^2 det G if `energy`.
+// that carries n's B); with G the node's record for pass C (interior nodes).
+// Returns the node's energy term zeta |B|^2 det G if `energy`.
 template <bool WITH_G>
 __device__ __forceinline__ double split_B_finish(const SplitArgs& a, int N, int n, int t, int i,
                                                  int j, int k, bool state, bool energy, int nw,
@@ -377,8 +376,9 @@ __global__ void __launch_bounds__(CURL == 2 ? DENSE_T2 : DENSE_T, 1) k_split_C(c
 //
 // One cooperative launch runs whole attempts: the twelve passes and the
 // step control, with no kernel boundary between them.  Each CTA keeps the
-// node ranges it has in the per-pass kernels (one CTA per SM, all resident), and instead of a grid-wide boundary after each pass
-// it waits only for the node planes its next pass reads:
+// node ranges it has in the per-pass kernels (one CTA per SM, all resident),
+// and instead of a grid-wide boundary after each pass it waits only for the
+// node planes its next pass reads:
 //   pass B of stage s at plane p reads the stage input at planes p-2..p+2,
 //     written by pass C of stage s-1 (the one-sided boundary stencil reaches
 //     two planes; the same wait orders pass C's earlier reads of the B, G

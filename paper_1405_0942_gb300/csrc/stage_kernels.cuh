@@ -1,6 +1,7 @@
 // Fused Cash-Karp stage kernels for the Lagrangian magneto-frictional step:
-// the direct current's in mixed precision, and the mimetic current's in FP64
-// where GLEMUR_F64_FUSED asks for it (the FP64 passes of kern_f64_split.cu and
+// the direct current's in mixed precision, and the mimetic current's in mixed
+// precision on rows of few 32-node tiles (kern_f32_narrow.cu) and in FP64 where
+// GLEMUR_F64_FUSED asks for it (the FP64 passes of kern_f64_split.cu and
 // kern_f64_direct.cu and the mixed mimetic march of stage_march.cuh are faster
 // for the rest; they share the arithmetic below).
 //
